@@ -13,12 +13,15 @@
 #include <complex>
 #include <cstdio>
 #include <cstring>
+#include <map>
+#include <mutex>
 #include <string>
 #include <vector>
 
 #include "zda.h"
 #include "zda_internal.h"
 #include "zda_step.h"
+#include "zda_resident.h"
 #include "zda_tile.h"
 
 using cd = std::complex<double>;
@@ -52,7 +55,7 @@ struct Layout {           // byte offsets inside the workspace
     size_t fields, psi_z, psi_r, psi_m, fields2, psi_h2, mon, des_f, des_a, rho_in, rho_bar, rho_t, rb, site_grad, g_t, g_rho,
         norm, src_rad, dft_hist, inv_r_n, inv_r_h, br_n, cr_n, br_h, cr_h, bm_n, cm_n, bm_h, cm_h, bz_n, cz_n, bz_h, cz_h, a_n, d_n, a_c, d_c, ph_n,
         ph_h, pulse, twiddle, adj_time, Gr, Gp, emph_n, emph_h, wt, beta_r, beta_p, g_in, partial, S,
-        umean, pt_row, qr, qw, qp, qwp, kk, energy, energy_part, status, total;
+        umean, pt_row, qr, qw, qp, qwp, kk, energy, energy_part, mail, status, total;
 };
 
 size_t align_up(size_t x) { return (x + 255) & ~size_t(255); }
@@ -89,7 +92,13 @@ struct zda_zone {
     zda::TileHMaps hmaps;           // tensor maps of the field buffer for the H half (variant 5)
     const char *hmaps_ws = nullptr;
     int hmaps_tj = 0;
-    int wait_limit = 1 << 22, inject_timeout = 0;   // bounded mbarrier waits of the fused step
+    // whole run in one launch (zda_resident.cu), the default where it fits; the plan is for r-PML form
+    // res_form (-1: not made yet)
+    zda::ResidentPlan res;
+    int res_form = -1;
+    size_t mail_bytes = 0;
+    bool grid_run = false;          // the last run's bricks waited on one another through memory
+    int wait_limit = 1 << 22, inject_timeout = 0;   // bounded waits of the fused, tiled and resident steps
     bool pair_kernels = true;       // split step: two z-cells per thread where the grid allows
     int rpml = 0;                   // r-PML form (zda_zone_set_radial_pml)
     int last_parity = 0;            // fused runs: which buffer holds the final fields
@@ -295,6 +304,7 @@ static void compute_layout(zda_zone &z)
     L.kk = take(Q * sizeof(double));
     L.energy = take(2 * T * sizeof(double));            // decay probe: W, Wdot per sample
     L.energy_part = take(2 * nr * sizeof(double));
+    L.mail = take(z.mail_bytes);                        // halo packets of the resident step
     L.status = take(sizeof(int) * 4);
     L.total = off;
 }
@@ -491,6 +501,28 @@ static zda_status upload(zda_zone &z)
     return ZDA_OK;
 }
 
+// the zone's cut for the resident step, for its present r-PML form
+static void make_resident_plan(zda_zone &z)
+{
+    if (z.res_form == z.rpml) return;
+    const zda_zone_desc &d = z.d;
+    zda::StepParams p{};
+    p.nr = d.n_r; p.nphi = d.n_phi; p.nz = d.n_z;
+    p.pr_in = d.pml_r_in; p.pr_out = d.pml_r_out; p.pz = d.pml_z;
+    p.bor = d.n_fold == 0 ? 1 : 0;
+    p.rpml_metric = z.rpml;
+    p.nq = z.nq;
+    int dev = 0, sms = 152, smem = 232448;
+    if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess ||
+        cudaDeviceGetAttribute(&smem, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev) != cudaSuccess) {
+        (void)cudaGetLastError();
+        sms = 152;
+        smem = 232448;
+    }
+    z.res = zda::resident_plan(p, sms, (size_t)smem);
+    z.res_form = z.rpml;
+}
+
 static zda_status derive(zda_zone &z)
 {
     const zda_zone_desc &d = z.d;
@@ -543,6 +575,9 @@ static zda_status derive(zda_zone &z)
     }
     if (z.variant == 1 && (d.n_z > zda::fused_max_nz() || bor)) z.variant = 0;
     if ((z.variant == 3 || z.variant == 4 || z.variant == 5) && (bor || d.n_z % 2 || d.pml_z % 2)) z.variant = 0;
+    z.res_form = -1;
+    make_resident_plan(z);
+    z.mail_bytes = z.res.blocks() ? zda::resident_mail_bytes(d.n_r, d.n_phi, d.n_z) : 0;
     compute_layout(z);
     z.tables_dirty = true;
     z.have_forward = false;
@@ -829,11 +864,75 @@ static zda_status tile_h_maps(zda_zone &z)
 }
 
 // kernels with bounded device-side waits report a timeout through the error word
-static bool uses_waits(const zda_zone &z) { return z.variant == 1 || z.variant >= 3; }
+static bool uses_waits(const zda_zone &z) { return z.variant == 1 || z.variant >= 3 || z.grid_run; }
 
-static zda_status time_loop(zda_zone &z, zda::StepParams &p, cudaStream_t s)
+// Whether this run takes the resident step; the launches of the split step
+// run instead under a kernel chosen by zda_zone_set_kernel, under the event
+// timing and the decay probe (both look between the launches of a step), and
+// where other work may run beside it (shared: a lens's branches, a stream
+// capture), because the resident step's blocks wait on one another.
+static bool resident_route(zda_zone &z, const zda::StepParams &p, bool shared)
+{
+    if (shared || !z.kernel_default || z.variant != 0 || z.time_every > 0 || !z.mail_bytes) return false;
+    if (z.probe_every > 0 && p.src_mode == zda::SRC_PLANE_WAVE) return false;
+    make_resident_plan(z);
+    return z.res.blocks() > 0;
+}
+
+// Two resident runs must not share the GPU (each would hold SMs that the
+// other's blocks wait for), so on every device each run's launches wait for
+// those of the run before, whatever their streams and threads.
+struct ResidentTurn {
+    std::mutex m;
+    cudaEvent_t last = nullptr;
+};
+static ResidentTurn &resident_turn(int device)
+{
+    static std::mutex m;
+    static std::map<int, ResidentTurn> turns;
+    std::lock_guard<std::mutex> g(m);
+    return turns[device];
+}
+
+// The whole run by the resident step; *done stays false where the device
+// cannot hold the grid at once (the launches of the split step run then).
+static zda_status resident_loop(zda_zone &z, zda::StepParams &p, cudaStream_t s, bool *done)
+{
+    p.dft_ne = zda::dft_entries(p);
+    void *mail = z.ws + z.L.mail;
+    CUDA_TRY(cudaMemsetAsync(mail, 0, z.mail_bytes, s));                     // no packet of an earlier run
+    ResidentTurn &turn = resident_turn(z.ctx->device);
+    std::lock_guard<std::mutex> guard(turn.m);
+    if (turn.last) CUDA_TRY(cudaStreamWaitEvent(s, turn.last, 0));
+    else CUDA_TRY(cudaEventCreateWithFlags(&turn.last, cudaEventDisableTiming));
+    // one launch per 4096 steps (a multiple of DFT_BLOCK): a run of any length stays preemptible
+    const int chunk = 4096;
+    for (int n = 0; n < z.d.n_steps; n += chunk) {
+        const cudaError_t e = zda::launch_resident(z.res, p, n, std::min(n + chunk, z.d.n_steps), z.d.n_steps, mail,
+                                                   P<int>(z, z.L.status) + 1, z.wait_limit, z.inject_timeout, s);
+        if (n == 0 && e == cudaErrorCooperativeLaunchTooLarge) {
+            (void)cudaGetLastError();
+            return ZDA_OK;
+        }
+        if (e != cudaSuccess) return fail(ZDA_ERR_CUDA, std::string("resident step: ") + cudaGetErrorString(e));
+        z.launches++;
+    }
+    CUDA_TRY(cudaEventRecord(turn.last, s));
+    z.grid_run = true;
+    z.last_parity = 0;
+    *done = true;
+    return ZDA_OK;
+}
+
+static zda_status time_loop(zda_zone &z, zda::StepParams &p, cudaStream_t s, bool shared)
 {
     const int R = (int)z.ev_pending.size();
+    z.grid_run = false;
+    if (resident_route(z, p, shared)) {
+        bool done = false;
+        const zda_status st = resident_loop(z, p, s, &done);
+        if (st || done) return st;
+    }
     if (z.variant == 3) {
         zda_status st = tile_maps(z);
         if (st) return st;
@@ -1026,7 +1125,7 @@ static zda_status focal(zda_zone &z, const float2 *mon, double *out_host, cudaSt
 
 // Everything of a forward run that is enqueued on the stream (no host sync):
 // filter + projection, cleared state, the time loop with DFTs, focal kernels.
-static zda_status forward_enqueue(zda_zone &z, const float *rho, cudaStream_t s)
+static zda_status forward_enqueue(zda_zone &z, const float *rho, cudaStream_t s, bool shared)
 {
     z.have_forward = false;
     zda_status st = run_filter(z, rho, s);
@@ -1042,7 +1141,7 @@ static zda_status forward_enqueue(zda_zone &z, const float *rho, cudaStream_t s)
     p.mon_k = z.d.monitor_k;
     p.mon = P<float2>(z, z.L.mon);
     p.des = P<float2>(z, z.L.des_f);
-    st = time_loop(z, p, s);
+    st = time_loop(z, p, s, shared);
     if (st) return st;
     z.probe_n = z.probe_every > 0 ? z.d.n_steps / z.probe_every : 0;
     return focal_enqueue(z, P<float2>(z, z.L.mon), s);
@@ -1050,7 +1149,7 @@ static zda_status forward_enqueue(zda_zone &z, const float *rho, cudaStream_t s)
 
 // Everything of an adjoint run that is enqueued (dI/dS already in g_in):
 // adjoint profiles, the adjoint time loop, overlap, transposed chain.
-static zda_status adjoint_enqueue(zda_zone &z, float *grad_rho, cudaStream_t s)
+static zda_status adjoint_enqueue(zda_zone &z, float *grad_rho, cudaStream_t s, bool shared)
 {
     const zda_zone_desc &d = z.d;
     const size_t plane = (size_t)d.n_r * d.n_phi;
@@ -1068,7 +1167,7 @@ static zda_status adjoint_enqueue(zda_zone &z, float *grad_rho, cudaStream_t s)
     p.mon_k = -1;
     p.mon = nullptr;
     p.des = P<float2>(z, z.L.des_a);
-    st = time_loop(z, p, s);
+    st = time_loop(z, p, s, shared);
     if (st) return st;
     zda::launch_site_gradient(P<float2>(z, z.L.des_f), P<float2>(z, z.L.des_a), P<float>(z, z.L.wt), z.nq,
                               d.n_r, d.n_phi, z.nk, d.r_lo, d.dr, vol, P<float>(z, z.L.site_grad), s);
@@ -1223,7 +1322,7 @@ zda_status zda_forward(zda_zone *z, const float *rho, double *focal_out, void *s
     if (st) return st;
     if (!rho || !focal_out) return fail(ZDA_ERR_ARG, "null pointer");
     cudaStream_t s = (cudaStream_t)stream;
-    st = forward_enqueue(*z, rho, s);
+    st = forward_enqueue(*z, rho, s, false);
     if (st) return st;
     st = check_wait_status(*z, s);
     if (st) return st;
@@ -1243,7 +1342,9 @@ zda_status zda_adjoint(zda_zone *z, const double *dI, float *grad_rho, void *str
         return fail(ZDA_ERR_ARG, "n_steps too short: the broadband adjoint pulses do not fit the run");
     cudaStream_t s = (cudaStream_t)stream;
     CUDA_TRY(cudaMemcpyAsync(z->ws + z->L.g_in, dI, z->nq * sizeof(double2), cudaMemcpyHostToDevice, s));
-    st = adjoint_enqueue(*z, grad_rho, s);
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    CUDA_TRY(cudaStreamIsCapturing(s, &cap));
+    st = adjoint_enqueue(*z, grad_rho, s, cap != cudaStreamCaptureStatusNone);
     if (st) return st;
     if (uses_waits(*z)) return check_wait_status(*z, s);
     return ZDA_OK;
@@ -1447,7 +1548,7 @@ zda_status zda_zone_time_steps(zda_zone *z, int steps, double *ms_out, void *str
     z->d.n_steps = steps;
     z->time_every = 0;
     cudaError_t e = cudaEventRecord(a, s);
-    if (e == cudaSuccess) st = time_loop(*z, p, s);
+    if (e == cudaSuccess) st = time_loop(*z, p, s, false);
     if (e == cudaSuccess && st == ZDA_OK) e = cudaEventRecord(b, s);
     if (e == cudaSuccess && st == ZDA_OK) e = cudaEventSynchronize(b);
     float ms = 0.f;
@@ -1581,7 +1682,7 @@ static size_t lens_ws_total(const zda_lens &L) { return lens_ws_status(L) + 256;
 static std::vector<long long> zone_stamp(const zda_zone &z)
 {
     return {(long long)(uintptr_t)z.ws, z.variant, z.pair_kernels, z.tile_phi, z.i_ranges, z.probe_every, z.d.n_steps, z.nq,
-            z.wait_limit, z.inject_timeout, (long long)z.lambda.size(), z.rpml};
+            z.wait_limit, z.inject_timeout, (long long)z.lambda.size(), z.rpml, z.kernel_default};
 }
 
 static bool stamps_match(const zda_lens &L, const std::vector<std::vector<long long>> &st)
@@ -1732,7 +1833,7 @@ zda_status zda_lens_forward(zda_lens *L, const float *const *rho, double *focal_
     int *status = (int *)(L->ws + lens_ws_status(*L));
     auto body = [&]() -> zda_status {
         zda_status st = lens_branches(*L, [&](zda_zone &Z, size_t, cudaStream_t sz) {
-            return forward_enqueue(Z, P<float>(Z, Z.L.rho_in), sz);
+            return forward_enqueue(Z, P<float>(Z, Z.L.rho_in), sz, true);
         });
         if (st) return st;
         CUDA_TRY(cudaMemsetAsync(status, 0, sizeof(int), L->streams[0]));
@@ -1781,7 +1882,7 @@ zda_status zda_lens_adjoint(zda_lens *L, const double *dI, float *const *grad_rh
     }
     auto body = [&]() -> zda_status {
         return lens_branches(*L, [&](zda_zone &Z, size_t, cudaStream_t sz) {
-            return adjoint_enqueue(Z, P<float>(Z, Z.L.g_rho), sz);
+            return adjoint_enqueue(Z, P<float>(Z, Z.L.g_rho), sz, true);
         });
     };
     zda_status st = lens_run(*L, L->g_adj, L->stamp_adj, s, body);
