@@ -259,7 +259,7 @@ static void compute_layout(zda_zone &z)
     L.g_t = take((size_t)z.nrd * np * sizeof(float));
     L.g_rho = take((size_t)z.nrd * np * sizeof(float));
     L.norm = take((size_t)z.nrd * sizeof(float));
-    L.src_rad = take(2 * nr * sizeof(float2));
+    L.src_rad = take((size_t)zda::DFT_BLOCK * 2 * nr * sizeof(float2));     // adjoint sources of DFT_BLOCK steps
     // history of the time-blocked DFT: design (3 components) + monitor (2) sites per slot
     L.dft_hist = take((size_t)zda::DFT_BLOCK * (3 * plane * z.nk + 2 * plane) * sizeof(float2));
     L.inv_r_n = take((nr + 1) * sizeof(float));
@@ -879,6 +879,18 @@ static bool resident_route(zda_zone &z, const zda::StepParams &p, bool shared)
     return z.res.blocks() > 0;
 }
 
+// Adjoint runs: the radial source of step n, worked out for DFT_BLOCK steps at
+// a time (a launch of its own per step cost 2-3 us of every step).
+static float2 *adjoint_source(zda_zone &z, const zda::StepParams &p, int n, cudaStream_t s)
+{
+    float2 *base = P<float2>(z, z.L.src_rad);
+    if (n % zda::DFT_BLOCK == 0) {
+        zda::launch_adjoint_source_rad(p, base, n, std::min(zda::DFT_BLOCK, z.d.n_steps - n), s);
+        z.launches++;
+    }
+    return base + (size_t)(n % zda::DFT_BLOCK) * 2 * z.d.n_r;
+}
+
 // Two resident runs must not share the GPU (each would hold SMs that the
 // other's blocks wait for), so on every device each run's launches wait for
 // those of the run before, whatever their streams and threads.
@@ -938,14 +950,14 @@ static zda_status time_loop(zda_zone &z, zda::StepParams &p, cudaStream_t s, boo
         if (st) return st;
         const bool dft = p.des || p.mon;
         p.dft_ne = zda::dft_entries(p);
-        const zda::TileParams tp[2] = {tile_params(z, p, 0), tile_params(z, p, 1)};
+        zda::TileParams tp[2] = {tile_params(z, p, 0), tile_params(z, p, 1)};
         const int nrc = tile_rchunks(z);
         const bool adj = p.src_mode == zda::SRC_ADJOINT;
         // timed samples: [tile step] between events 0 and 1, [DFT flush] between 2 and 3
         for (int n = 0; n < z.d.n_steps; ++n) {
             const bool timed = z.time_every > 0 && R > 0 && (n % z.time_every) == z.time_every - 1;
             int slot = 0;
-            if (adj) zda::launch_adjoint_source_rad(p, n, s);
+            if (adj) tp[n & 1].p.src_rad = adjoint_source(z, p, n, s);
             if (timed) {
                 slot = z.ev_next;
                 z.ev_next = (z.ev_next + 1) % R;
@@ -970,7 +982,7 @@ static zda_status time_loop(zda_zone &z, zda::StepParams &p, cudaStream_t s, boo
             }
         }
         z.last_parity = z.d.n_steps & 1;
-        z.launches += (long long)z.d.n_steps * (adj ? 2 : 1);
+        z.launches += (long long)z.d.n_steps;
         CUDA_TRY(cudaGetLastError());
         return ZDA_OK;
     }
@@ -1038,7 +1050,7 @@ static zda_status time_loop(zda_zone &z, zda::StepParams &p, cudaStream_t s, boo
     for (int n = 0; n < z.d.n_steps; ++n) {
         const bool timed = z.time_every > 0 && R > 0 && (n % z.time_every) == z.time_every - 1;
         int slot = 0;
-        if (pair && p.src_mode == zda::SRC_ADJOINT) zda::launch_adjoint_source_rad(p, n, s);
+        if (pair && p.src_mode == zda::SRC_ADJOINT) etp.p.src_rad = p.src_rad = adjoint_source(z, p, n, s);
         if (timed) {
             slot = z.ev_next;
             z.ev_next = (z.ev_next + 1) % R;
@@ -1077,7 +1089,6 @@ static zda_status time_loop(zda_zone &z, zda::StepParams &p, cudaStream_t s, boo
             z.ev_pending[slot] = 1;
         }
     }
-    if (pair) z.launches += (long long)z.d.n_steps * (p.src_mode == zda::SRC_ADJOINT ? 1 : 0);
     z.launches += 2LL * z.d.n_steps;
     CUDA_TRY(cudaGetLastError());
     return ZDA_OK;

@@ -120,7 +120,7 @@ constexpr int DFT_BLOCK = 32;
 size_t dft_entries(const StepParams &p);
 bool dft_flush_due(const StepParams &p, int n, int n_steps);
 void launch_dft_flush(const StepParams &p, int n, cudaStream_t s);
-void launch_adjoint_source_rad(const StepParams &p, int n, cudaStream_t s);
+void launch_adjoint_source_rad(const StepParams &p, float2 *out, int n, int steps, cudaStream_t s);   // [steps][2][n_r]
 
 struct FilterParams {
     int nrd, nphi, di_max, dj_max;

@@ -423,25 +423,27 @@ void launch_dft_flush(const StepParams &p, int n, cudaStream_t s)
     k_dft_flush<<<(unsigned)((nsites + 255) / 256), 256, 0, s>>>(p, nslots, n - (nslots - 1));
 }
 
-// Adjoint source of step n per radius: sum_q beta_q(r) k_q(t_{n+1/2}) for the
-// E_r and E_phi sites (the e^{i phi} factor is applied per row).
-__global__ void k_adjoint_source_rad(const StepParams p, const int n)
+// Adjoint sources of `steps` steps from n on, per radius: sum_q beta_q(r)
+// k_q(t_{n+1/2}) for the E_r and E_phi sites (the e^{i phi} factor is applied
+// per row).
+__global__ void k_adjoint_source_rad(const StepParams p, float2 *out, const int n)
 {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= p.nr) return;
-    const float2 *kt = p.t.adj_time + (size_t)n * p.nq;
+    const float2 *kt = p.t.adj_time + (size_t)(n + blockIdx.y) * p.nq;
     float2 sr = make_float2(0.f, 0.f), sp = make_float2(0.f, 0.f);
     for (int q = 0; q < p.nq; ++q) {
         sr = c_fma(p.beta_r[(size_t)q * p.nr + i], kt[q], sr);
         sp = c_fma(p.beta_p[(size_t)q * p.nr + i], kt[q], sp);
     }
-    p.src_rad[i] = sr;
-    p.src_rad[p.nr + i] = sp;
+    out += (size_t)blockIdx.y * 2 * p.nr;
+    out[i] = sr;
+    out[p.nr + i] = sp;
 }
 
-void launch_adjoint_source_rad(const StepParams &p, int n, cudaStream_t s)
+void launch_adjoint_source_rad(const StepParams &p, float2 *out, int n, int steps, cudaStream_t s)
 {
-    k_adjoint_source_rad<<<(p.nr + 127) / 128, 128, 0, s>>>(p, n);
+    k_adjoint_source_rad<<<dim3((p.nr + 127) / 128, steps), 128, 0, s>>>(p, out, n);
 }
 
 bool pair_kernels_apply(const StepParams &p) { return p.nz % 2 == 0 && p.pz % 2 == 0 && !p.bor; }
