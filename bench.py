@@ -65,7 +65,7 @@ def parse():
                     help="radius ranges of the tile kernels chosen by --kernel (0: the library's rule)")
     ap.add_argument("--kernel", default="default",
                     choices=["default", "split", "split1", "fused2", "fused4", "tile4", "tile8", "tile16", "etile8",
-                             "etile16", "etile32", "htile8", "htile16", "htile32", "tuned"],
+                             "etile16", "etile32", "htile8", "htile16", "htile32", "two8", "two16", "tuned"],
                     help="time-step kernel (default: the library's choice for the zone; tuned: the tile tuner's "
                          "pick)")
     return ap.parse_args()
@@ -78,10 +78,10 @@ def whole_step(gcells_per_gpu, peak_gbs, kernels, per_step):
     """The whole step against the HBM roofline: frac_96B = Gcell-upd/s x 96 B
     (one read and one write of the six field components, the one-step
     minimum) / peak; frac_step_bytes = the step kernels' algorithmic bytes
-    per step (the DFT flush's per launch / 32) / their summed event time per
+    per step (the DFT flush's per launch / 32, the two-step kernel's / 2) / their summed event time per
     step / peak.  kernels: (name, bytes per launch, ms per launch);
     per_step: name -> ms per step."""
-    step_bytes = sum(b / 32 if nm == "k_dft_flush" else b for nm, b, _ in kernels)
+    step_bytes = sum(b / {"k_dft_flush": 32, "k_two": 2}.get(nm, 1) for nm, b, _ in kernels)
     step_ms = sum(per_step.values())
     return {"frac_96B": gcells_per_gpu * 96.0 / peak_gbs,
             "algorithmic_bytes_per_step": step_bytes, "kernel_ms_per_step": step_ms,
@@ -93,7 +93,8 @@ def kernel_choice(a):
     k = {"split": (0, 16, 0), "split1": (2, 2, 0), "fused2": (1, 2, 0), "fused4": (1, 4, 0),
          "tile4": (3, 4, 0), "tile8": (3, 8, 0), "tile16": (3, 16, 0),
          "etile8": (4, 8, 0), "etile16": (4, 16, 0), "etile32": (4, 32, 0),
-         "htile8": (5, 8, 0), "htile16": (5, 16, 0), "htile32": (5, 32, 0)}.get(a.kernel)
+         "htile8": (5, 8, 0), "htile16": (5, 16, 0), "htile32": (5, 32, 0),
+         "two8": (6, 8, 0), "two16": (6, 16, 0)}.get(a.kernel)
     if k is not None and k[0] >= 3 and a.tile_ranges > 0:
         k = (k[0], k[1], a.tile_ranges)
     return k
@@ -413,6 +414,9 @@ def run_ours(a):
     elif variant == 3:
         # the fused tile step also writes the DFT history (8 B per DFT site); the flush is timed below
         kernels = [("k_tile_step", algorithmic_bytes_stream(spec) + dft_entries(spec) * 8, avg[0])]
+    elif variant == 6:
+        # one launch reads and writes the state once for two steps, and writes the DFT history of both
+        kernels = [("k_two", algorithmic_bytes_stream(spec) + dft_entries(spec) * 16, avg[0])]
     elif pair:
         # the DFT history is written by the E update; the flush (every 32 steps)
         # is timed on its own below
@@ -422,8 +426,8 @@ def run_ours(a):
     else:
         kernels = [("k_update_h", algorithmic_bytes_h(spec, rpml), avg[0]),
                    ("k_update_e", algorithmic_bytes_e(spec, nq, rpml=rpml), avg[1])]
-    per_step = {nm: t for nm, _, t in kernels}
-    if pair or variant == 3:
+    per_step = {nm: t / 2 if nm == "k_two" else t for nm, _, t in kernels}
+    if pair or variant in (3, 6):
         kernels.append(("k_dft_flush", algorithmic_bytes_dft_flush(spec, nq), avg[2]))
         per_step["k_dft_flush"] = avg[2] / 32                # one flush per 32 steps
     kernels.sort(key=lambda k: -per_step[k[0]])            # dominant (most GPU time per step) first
@@ -452,7 +456,8 @@ def run_ours(a):
                                         2: "split, one z-cell per thread",
                                         3: "fused, TMA-staged tiles streaming along r",
                                         4: "split, E half on TMA-staged tiles streaming along r",
-                                        5: "split, both halves on TMA-staged tiles streaming along r"}[variant],
+                                        5: "split, both halves on TMA-staged tiles streaming along r",
+                                        6: "two steps per launch, tiles streaming along r"}[variant],
                             "tile_phi": tile_phi,
                             "i_ranges": i_ranges, "radial_pml": zone.radial_pml()},
             "e2e": e2e, "gpu_launches": launches, "clocks": clk,

@@ -233,13 +233,23 @@ long long zda_zone_launch_count(const zda_zone *zone);
  * even n_z and pml_z, real-radius r-PML): one fused launch per step on
  * tiles of tile_phi in {4, 8, 16} phi rows x 32 z-cells staged by TMA, each
  * thread block streaming over one of i_ranges radius ranges (0 = about 21
- * radii each).  Default at zone creation: variant 4 with 16 rows where it
- * applies and the zone gives at least four waves of its thread blocks (2 per
- * SM) in radius ranges of about 21 radii, else variant 0; selecting
+ * radii each).  variant 6 (annular zones, even n_z >= 4 and even pml_z,
+ * real-radius r-PML): one launch per two steps on tiles of at most tile_phi
+ * in {4, 8, 16} phi rows streaming over one of i_ranges radius ranges (0 =
+ * by a cost rule), ping-pong buffers; a run under the decay probe takes the
+ * split step.  Default at zone creation: variant 6 with 16 rows where it
+ * applies and the zone has at least 2.2 million cells and 128 radii; else
+ * variant 4 with 16 rows where it applies and the zone gives at least four
+ * waves of its thread blocks (2 per SM) in radius ranges of about 21 radii;
+ * else variant 0.  A zone with the default variant 0 whose whole field state
+ * fits in the registers of one grid runs all its steps in one launch
+ * instead (not under zda_zone_set_timing or the decay probe, and not where
+ * zones of a lens share the GPU).  Selecting
  * the stretched r-PML (form 1) on a zone that still has the default falls
- * back to variant 0, while an explicit variant 1, 3 or 4 refuses it.  All
+ * back to variant 0, while an explicit variant 1, 3, 4, 5 or 6 refuses it.  All
  * compute the same scheme; results agree to FP32 rounding.  Variants 1, 3
- * and 4 bound their device-side waits (zda_zone_set_wait_limit). */
+ * to 5 and the one-launch run bound their device-side waits
+ * (zda_zone_set_wait_limit). */
 zda_status zda_zone_set_kernel(zda_zone *zone, int variant, int tile_phi, int i_ranges);
 zda_status zda_zone_get_kernel(const zda_zone *zone, int *variant, int *tile_phi, int *i_ranges);
 
@@ -259,7 +269,7 @@ zda_status zda_zone_get_kernel(const zda_zone *zone, int *variant, int *tile_phi
  *   Reflection of a cylindrical pulse at w0, against a radially larger
  *   domain: 1.9e-3 (form 0) vs 5e-5 (form 1) at r = 10 lambda.
  * Form 1 runs on the split step (variants 0 and 2); the fused steps
- * (variants 1 and 3) refuse it (ZDA_ERR_ARG either way round).  Takes effect at
+ * (variants 1 and 3) and the tiled ones (4 to 6) refuse it (ZDA_ERR_ARG either way round).  Takes effect at
  * the next run; a zda_adjoint needs a zda_forward of the same form. */
 zda_status zda_zone_set_radial_pml(zda_zone *zone, int form);
 zda_status zda_zone_get_radial_pml(const zda_zone *zone, int *form);
@@ -270,9 +280,10 @@ zda_status zda_zone_get_radial_pml(const zda_zone *zone, int *form);
  * zda_adjoint needs a new zda_forward).  Used by the tile-shape tuner. */
 zda_status zda_zone_time_steps(zda_zone *zone, int steps, double *ms_out_host, void *stream);
 
-/* The fused and tiled steps (variants 1, 3, 4) wait on shared-memory
- * barriers for their staged copies; every wait gives up after `polls` polls
- * (default 4194304; variants 3 and 4 also after one second), sets an error
+/* The fused and tiled steps (variants 1, 3, 4, 5) wait on shared-memory
+ * barriers for their staged copies, the one-launch run of a small zone on
+ * its neighbour blocks' halos; every wait gives up after `polls` polls
+ * (default 4194304; variants 3 to 5 also after one second), sets an error
  * word and lets the kernel finish, and the call then returns
  * ZDA_ERR_TIMEOUT (zda_forward, zda_adjoint and zda_iteration synchronise
  * their stream to read it).  inject_timeout != 0 is for tests of that path:
@@ -291,7 +302,9 @@ zda_status zda_zone_set_wait_limit(zda_zone *zone, int polls, int inject_timeout
  * writes the DFT history), DFT flush (only on steps 31, 63, ...: sample
  * with every = 32 to time it);
  * split step with one z-cell per thread: H update, E update (with the DFTs), -;
- * fused step: streaming E/H kernel, -, DFT kernel ("-" reads 0). */
+ * fused step: streaming E/H kernel, -, DFT kernel ("-" reads 0);
+ * two-step form: the launch of the sampled step and its neighbour, -, DFT
+ * flush (one sample per launch: every = 1 samples each pair of steps once). */
 zda_status zda_zone_set_timing(zda_zone *zone, int every);
 zda_status zda_zone_timing(zda_zone *zone, double *ms3_host, long long *count_host);
 

@@ -23,6 +23,7 @@
 #include "zda_step.h"
 #include "zda_resident.h"
 #include "zda_tile.h"
+#include "zda_two.h"
 
 using cd = std::complex<double>;
 
@@ -52,7 +53,7 @@ struct zda_ctx {
 namespace {
 
 struct Layout {           // byte offsets inside the workspace
-    size_t fields, psi_z, psi_r, psi_m, fields2, psi_h2, mon, des_f, des_a, rho_in, rho_bar, rho_t, rb, site_grad, g_t, g_rho,
+    size_t fields, psi_z, psi_r, psi_m, fields2, psi_h2, psi_e2, mon, des_f, des_a, rho_in, rho_bar, rho_t, rb, site_grad, g_t, g_rho,
         norm, src_rad, dft_hist, inv_r_n, inv_r_h, br_n, cr_n, br_h, cr_h, bm_n, cm_n, bm_h, cm_h, bz_n, cz_n, bz_h, cz_h, a_n, d_n, a_c, d_c, ph_n,
         ph_h, pulse, twiddle, adj_time, Gr, Gp, emph_n, emph_h, wt, beta_r, beta_p, g_in, partial, S,
         umean, pt_row, qr, qw, qp, qwp, kk, energy, energy_part, mail, status, total;
@@ -80,7 +81,8 @@ struct zda_zone {
     // streaming along r (bulk-copy ring), 3 = fused single launch on TMA-staged
     // tiles (tile_phi rows x 32 z-cells, streaming over i_ranges radius ranges), 4 = split
     // step with the E half on TMA-staged tiles (tile_phi rows, i_ranges radius ranges), 5 = split
-    // step with both halves on those tiles
+    // step with both halves on those tiles, 6 = two steps per launch on tiles (at most tile_phi
+    // rows, i_ranges radius ranges)
     int variant = 0, tile_phi = 2, i_ranges = 0;
     zda::TileMaps tmaps[2];         // tensor maps of the two field buffers (variant 3)
     const char *tmaps_ws = nullptr; // the workspace and tile shape they were encoded for
@@ -245,9 +247,10 @@ static void compute_layout(zda_zone &z)
     L.psi_z = take(4 * plane * 2 * d.pml_z * sizeof(float2));
     L.psi_r = take(4 * (size_t)(d.pml_r_in + d.pml_r_out) * np * nz * sizeof(float2));
     L.psi_m = take(4 * (size_t)(d.pml_r_in + d.pml_r_out) * np * nz * sizeof(float2));   // zeroed with psi_r
-    // second field buffer and H-side CPML set for the fused (ping-pong) step
+    // second field buffer and CPML sets for the fused and two-step (ping-pong) forms
     L.fields2 = take(6 * ncell * sizeof(float2));
     L.psi_h2 = take((2 * plane * 2 * d.pml_z + 2 * (size_t)(d.pml_r_in + d.pml_r_out) * np * nz) * sizeof(float2));
+    L.psi_e2 = take((2 * plane * 2 * d.pml_z + 2 * (size_t)(d.pml_r_in + d.pml_r_out) * np * nz) * sizeof(float2));
     L.mon = take(Q * 2 * plane * sizeof(float2));
     L.des_f = take(Q * 3 * plane * z.nk * sizeof(float2));
     L.des_a = take(Q * 3 * plane * z.nk * sizeof(float2));
@@ -574,7 +577,7 @@ static zda_status derive(zda_zone &z)
         z.di_max = z.dj_max = 0;
     }
     if (z.variant == 1 && (d.n_z > zda::fused_max_nz() || bor)) z.variant = 0;
-    if ((z.variant == 3 || z.variant == 4 || z.variant == 5) && (bor || d.n_z % 2 || d.pml_z % 2)) z.variant = 0;
+    if (z.variant >= 3 && (bor || d.n_z % 2 || d.pml_z % 2)) z.variant = 0;
     z.res_form = -1;
     make_resident_plan(z);
     z.mail_bytes = z.res.blocks() ? zda::resident_mail_bytes(d.n_r, d.n_phi, d.n_z) : 0;
@@ -864,7 +867,7 @@ static zda_status tile_h_maps(zda_zone &z)
 }
 
 // kernels with bounded device-side waits report a timeout through the error word
-static bool uses_waits(const zda_zone &z) { return z.variant == 1 || z.variant >= 3 || z.grid_run; }
+static bool uses_waits(const zda_zone &z) { return z.variant == 1 || (z.variant >= 3 && z.variant <= 5) || z.grid_run; }
 
 // Whether this run takes the resident step; the launches of the split step
 // run instead under a kernel chosen by zda_zone_set_kernel, under the event
@@ -889,6 +892,119 @@ static float2 *adjoint_source(zda_zone &z, const zda::StepParams &p, int n, cuda
         z.launches++;
     }
     return base + (size_t)(n % zda::DFT_BLOCK) * 2 * z.d.n_r;
+}
+
+// tile rows and radius ranges of the two-step form (0: chosen by two_plan)
+static zda::TwoPlan two_step_plan(const zda_zone &z)
+{
+    zda::StepParams p{};
+    p.nr = z.d.n_r; p.nphi = z.d.n_phi; p.nz = z.d.n_z;
+    p.pr_in = z.d.pml_r_in; p.pr_out = z.d.pml_r_out; p.pz = z.d.pml_z;
+    p.bor = z.d.n_fold == 0 ? 1 : 0;
+    p.rpml_metric = z.rpml;
+    int dev = 0, sms = 152, smem = 232448;
+    if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess ||
+        cudaDeviceGetAttribute(&smem, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev) != cudaSuccess) {
+        (void)cudaGetLastError();
+        sms = 152;
+        smem = 232448;
+    }
+    return zda::two_plan(p, z.tile_phi, std::min(z.i_ranges, z.d.n_r), sms, (size_t)smem);
+}
+
+// Whether the split step of a default zone runs its E update on TMA tiles of 16 phi rows: annular, even n_z
+// and z-PML, and at least four waves of thread blocks (2 per SM) in radius ranges of about 21 radii.  Slower
+// on zones of 16 or fewer phi cells and on the 200-phi-cell zones of the 40-zone lens, where ranges get short.
+static bool split_takes_tiles(const zda_zone_desc &d)
+{
+    if (d.n_fold == 0 || d.n_z % 2 || d.pml_z % 2) return false;
+    int dev = 0, sms = 152;
+    if (cudaGetDevice(&dev) != cudaSuccess ||
+        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) {
+        (void)cudaGetLastError();
+        sms = 152;
+    }
+    const long long tiles = (long long)((d.n_z + 31) / 32) * ((d.n_phi + 15) / 16);
+    return tiles * (d.n_r / 21) >= 8LL * sms;
+}
+
+// A run by the two-step form: state and CPML auxiliaries change buffers with
+// every launch; a last odd step is a split step on the buffer it finds.
+static zda_status two_step_loop(zda_zone &z, zda::StepParams &p, cudaStream_t s)
+{
+    using namespace zda;
+    const zda_zone_desc &d = z.d;
+    const size_t ncell = (size_t)d.n_r * d.n_phi * d.n_z;
+    const size_t nzs = (size_t)d.n_r * d.n_phi * 2 * d.pml_z, nrs = (size_t)(d.pml_r_in + d.pml_r_out) * d.n_phi * d.n_z;
+    const TwoPlan pl = two_step_plan(z);
+    if (!pl.ranges) return fail(ZDA_ERR_ARG, "the two-step form does not fit this zone");
+    const bool dft = p.des || p.mon, adj = p.src_mode == SRC_ADJOINT;
+    p.dft_ne = dft_entries(p);
+    float2 *F[2] = {P<float2>(z, z.L.fields), P<float2>(z, z.L.fields2)};
+    float2 *h2 = P<float2>(z, z.L.psi_h2), *e2 = P<float2>(z, z.L.psi_e2);
+    float2 *ps[2][PS_N] = {{p.psi.hr_z, p.psi.hp_z, p.psi.er_z, p.psi.ep_z, p.psi.hp_r, p.psi.hz_r, p.psi.ep_r, p.psi.ez_r},
+                           {h2, h2 + nzs, e2, e2 + nzs, h2 + 2 * nzs, h2 + 2 * nzs + nrs, e2 + 2 * nzs, e2 + 2 * nzs + nrs}};
+    TwoParams tp[2];
+    for (int b = 0; b < 2; ++b) {
+        tp[b] = TwoParams{};
+        tp[b].p = p;
+        for (int c = 0; c < 3; ++c) {
+            tp[b].iE[c] = F[b] + c * ncell;
+            tp[b].iH[c] = F[b] + (3 + c) * ncell;
+            tp[b].oE[c] = F[1 - b] + c * ncell;
+            tp[b].oH[c] = F[1 - b] + (3 + c) * ncell;
+        }
+        for (int c = 0; c < PS_N; ++c) {
+            tp[b].iP[c] = ps[b][c];
+            tp[b].oP[c] = ps[1 - b][c];
+        }
+    }
+    const int R = (int)z.ev_pending.size();
+    int b = 0;
+    // timed samples: [two steps] between events 0 and 1, [DFT flush] between 2 and 3
+    for (int n = 0; n < d.n_steps; n += 2) {
+        const int last = std::min(n + 1, d.n_steps - 1);
+        const bool timed = z.time_every > 0 && R > 0 && (n / z.time_every != (last + 1) / z.time_every);
+        int slot = 0;
+        float2 *src = adj ? adjoint_source(z, p, n, s) : nullptr;
+        if (timed) {
+            slot = z.ev_next;
+            z.ev_next = (z.ev_next + 1) % R;
+            timing_drain_slot(z, slot);
+            CUDA_TRY(cudaEventRecord(z.ev[4 * slot], s));
+        }
+        if (last > n) {
+            tp[b].p.src_rad = src;
+            const cudaError_t e = launch_two(pl, tp[b], n, s);
+            if (e != cudaSuccess) return fail(ZDA_ERR_CUDA, std::string("two-step tile kernel: ") + cudaGetErrorString(e));
+            z.launches++;
+            b ^= 1;
+        } else {                                   // the odd last step, in place
+            StepParams o = p;
+            o.f = Fields{F[b], F[b] + ncell, F[b] + 2 * ncell, F[b] + 3 * ncell, F[b] + 4 * ncell, F[b] + 5 * ncell};
+            o.psi = Psi{ps[b][PS_HR_Z], ps[b][PS_HP_Z], ps[b][PS_HP_R], ps[b][PS_HZ_R],
+                        ps[b][PS_ER_Z], ps[b][PS_EP_Z], ps[b][PS_EP_R], ps[b][PS_EZ_R]};
+            o.src_rad = src;
+            launch_update_h_pair(o, s);
+            launch_update_e_pair(o, n, s);
+            z.launches += 2;
+        }
+        if (timed) {
+            CUDA_TRY(cudaEventRecord(z.ev[4 * slot + 1], s));
+            CUDA_TRY(cudaEventRecord(z.ev[4 * slot + 2], s));
+        }
+        if (dft && dft_flush_due(p, last, d.n_steps)) {
+            launch_dft_flush(p, last, s);
+            z.launches++;
+        }
+        if (timed) {
+            CUDA_TRY(cudaEventRecord(z.ev[4 * slot + 3], s));
+            z.ev_pending[slot] = 1;
+        }
+    }
+    z.last_parity = b;
+    CUDA_TRY(cudaGetLastError());
+    return ZDA_OK;
 }
 
 // Two resident runs must not share the GPU (each would hold SMs that the
@@ -945,6 +1061,8 @@ static zda_status time_loop(zda_zone &z, zda::StepParams &p, cudaStream_t s, boo
         const zda_status st = resident_loop(z, p, s, &done);
         if (st || done) return st;
     }
+    // (the decay probe compares the states around a step: it takes the split step)
+    if (z.variant == 6 && !(z.probe_every > 0 && p.src_mode == zda::SRC_PLANE_WAVE)) return two_step_loop(z, p, s);
     if (z.variant == 3) {
         zda_status st = tile_maps(z);
         if (st) return st;
@@ -1025,7 +1143,8 @@ static zda_status time_loop(zda_zone &z, zda::StepParams &p, cudaStream_t s, boo
     const bool dft = pair && (p.des || p.mon);
     p.dft_ne = zda::dft_entries(p);
     if (!pair) p.dft_hist = nullptr;
-    const bool etile = pair && (z.variant == 4 || z.variant == 5), htile = pair && z.variant == 5;
+    const bool etile = pair && (z.variant == 4 || z.variant == 5 ||
+                                (z.variant == 6 && z.kernel_default && split_takes_tiles(z.d))), htile = pair && z.variant == 5;
     zda::TileParams etp{};
     int enrc = 1;
     if (etile) {
@@ -1216,24 +1335,19 @@ zda_status zda_zone_create(zda_ctx *ctx, const zda_zone_desc *desc, zda_zone **o
     zda_zone *z = new zda_zone();
     z->ctx = ctx;
     z->d = *desc;
-    // default step: split H update + E update on TMA tiles of 16 phi rows where the zone allows
-    // (annular, even n_z and z-PML) and is large enough for them: at least four waves of thread
-    // blocks (2 per SM) in radius ranges of about 21 radii.  Measured on GB300: 8 % faster per step
-    // than the thread-per-pair E update on the 300 x 320 x 160 wide zone; slower on zones of 16 or
-    // fewer phi cells and on the 200-phi-cell zones of the 40-zone lens, where the ranges get short.
-    if (desc->n_fold > 0 && desc->n_z % 2 == 0 && desc->pml_z % 2 == 0) {
-        int dev = 0, sms = 152;
-        if (cudaGetDevice(&dev) != cudaSuccess ||
-            cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) {
-            (void)cudaGetLastError();
-            sms = 152;
-        }
-        const long long tiles = (long long)((desc->n_z + 31) / 32) * ((desc->n_phi + 15) / 16);
-        if (tiles * (desc->n_r / 21) >= 8LL * sms) {
-            z->variant = 4;
-            z->tile_phi = 16;
-        }
+    // default step, on zones too large for the resident step (annular, even n_z and z-PML).  Two steps per
+    // launch on tiles of 16 phi rows from 2.2 M cells on, if there are 128 radii to stream over; else the
+    // split step (split_takes_tiles).  Measured on GB300, us per step, two-step | split (the
+    // better of its forms): 300 x 320 x 160 cells 330 | 391; 144 x 128 x 160 81 | 93; 157 x 96 x 160 62 | 77;
+    // 216 x 114 x 112 84 | 94; below the line 208 x 48 x 160 49 | 44; 123 x 95 x 62 33 | 25; 916 x 16 x 100
+    // 48 | 43; and with few radii 60 x 320 x 160 107 | 99.
+    if (desc->n_fold > 0 && desc->n_r >= 128 && (double)desc->n_r * desc->n_phi * desc->n_z >= 2.2e6) {
+        z->variant = 6;
+        z->tile_phi = 16;
+        if (!two_step_plan(*z).ranges) z->variant = 0;
     }
+    if (z->variant == 0 && split_takes_tiles(*desc)) z->variant = 4;
+    z->tile_phi = z->variant ? 16 : 2;
     zda_status st = derive(*z);
     if (st != ZDA_OK) { delete z; return st; }
     *out = z;
@@ -1435,7 +1549,7 @@ zda_status zda_copy_fields(zda_zone *z, float *out, void *stream)
     if (st) return st;
     if (!out) return fail(ZDA_ERR_ARG, "null pointer");
     const size_t n = 6 * (size_t)z->d.n_r * z->d.n_phi * z->d.n_z * sizeof(float2);
-    const size_t off = ((z->variant == 1 || z->variant == 3) && z->last_parity) ? z->L.fields2 : z->L.fields;
+    const size_t off = ((z->variant == 1 || z->variant == 3 || z->variant == 6) && z->last_parity) ? z->L.fields2 : z->L.fields;
     CUDA_TRY(cudaMemcpyAsync(out, z->ws + off, n, cudaMemcpyDeviceToDevice, (cudaStream_t)stream));
     return ZDA_OK;
 }
@@ -1465,8 +1579,27 @@ long long zda_zone_launch_count(const zda_zone *z) { return z ? z->launches : -1
 
 zda_status zda_zone_set_kernel(zda_zone *z, int variant, int tile_phi, int i_ranges)
 {
-    if (!z || variant < 0 || variant > 5 || i_ranges < 0) return fail(ZDA_ERR_ARG, "bad kernel choice");
+    if (!z || variant < 0 || variant > 6 || i_ranges < 0) return fail(ZDA_ERR_ARG, "bad kernel choice");
     z->kernel_default = false;
+    if (variant == 6) {                      // two steps per launch on tiles streaming along r
+        if (z->d.n_fold == 0) return fail(ZDA_ERR_ARG, "the axis zone (continuous axisymmetry) uses the split step");
+        if (z->rpml) return fail(ZDA_ERR_ARG, "the two-step form implements the real-radius r-PML only");
+        if (z->d.n_z % 2 || z->d.pml_z % 2) return fail(ZDA_ERR_ARG, "the two-step form needs even n_z and pml_z");
+        if (tile_phi != 4 && tile_phi != 8 && tile_phi != 16)
+            return fail(ZDA_ERR_ARG, "two-step form: tile_phi must be 4, 8 or 16");
+        zda_zone t;
+        t.d = z->d;
+        t.tile_phi = tile_phi;
+        t.i_ranges = i_ranges;
+        if (!two_step_plan(t).ranges)
+            return fail(ZDA_ERR_ARG, "two-step form: n_z is below 4, or a radius range does not fit in shared memory");
+        z->pair_kernels = true;
+        z->variant = variant;
+        z->tile_phi = tile_phi;
+        z->i_ranges = i_ranges;
+        z->have_forward = false;
+        return ZDA_OK;
+    }
     if (variant == 4 || variant == 5) {      // split step, E half (4) or both halves (5) on TMA-staged tiles
         if (z->d.n_fold == 0) return fail(ZDA_ERR_ARG, "the axis zone (continuous axisymmetry) uses the split step");
         if (z->rpml) return fail(ZDA_ERR_ARG, "the E tile kernel implements the real-radius r-PML only");
@@ -1589,6 +1722,7 @@ zda_status zda_zone_get_kernel(const zda_zone *z, int *variant, int *tile_phi, i
     *tile_phi = z->tile_phi;
     *i_ranges = z->variant == 1   ? auto_i_ranges(*z)
                 : z->variant == 3 ? tile_rchunks(*z)
+                : z->variant == 6 ? two_step_plan(*z).ranges
                 : z->variant >= 4 ? tile_e_rchunks(*z)
                                   : z->i_ranges;
     return ZDA_OK;

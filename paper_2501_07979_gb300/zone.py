@@ -204,7 +204,9 @@ class Zone:
         rows per block), 1 fused streaming (tile_phi 2 or 4), 2 split one cell
         per thread, 3 fused TMA tiles (tile_phi 4, 8 or 16; i_ranges radius
         ranges), 4 split with the E half on TMA tiles (tile_phi 8, 16 or 32;
-        i_ranges radius ranges), 5 the same with both halves on TMA tiles."""
+        i_ranges radius ranges), 5 the same with both halves on TMA tiles,
+        6 two steps per launch (at most tile_phi = 4, 8 or 16 phi rows per
+        tile; i_ranges radius ranges)."""
         check(_lib.lib().zda_zone_set_kernel(self.handle, int(variant), int(tile_phi), int(i_ranges)))
 
     def set_radial_pml(self, form):
@@ -243,7 +245,8 @@ class Zone:
         """([ms of launch 1, 2, 3 summed over the samples], sampled steps) since
         the last call; split step: H update, E update, DFT update (one z-cell
         per thread: the DFT is inside the E update); fused step: streaming
-        kernel, 0, DFT kernel."""
+        kernel, 0, DFT kernel; two-step form: the launch of the sampled step
+        and its neighbour, 0, DFT flush."""
         ms = (ctypes.c_double * 3)()
         n = ctypes.c_longlong()
         check(_lib.lib().zda_zone_timing(self.handle, ms, ctypes.byref(n)))
