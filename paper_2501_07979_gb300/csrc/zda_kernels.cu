@@ -23,6 +23,8 @@
 // 1/r_0 is 0, so H_r(0) keeps its value 0; E_z(0) and E_phi(0) are not
 // updated (E_z vanishes on the axis for |m| = 1 and E_phi(0), H_r(0) enter the
 // other updates multiplied by r = 0).
+#include <cooperative_groups.h>
+
 #include "zda_internal.h"
 
 namespace zda {
@@ -609,25 +611,51 @@ void launch_focal_sum(const double2 *partial, int nq, int nr, double2 *S, int *s
 // imaginary), divided by `scale`.  S[b][q] = sum_i Gr_q(i) sum_j emph_n(j) E_r
 // + Gp_q(i) sum_j emph_h(j) E_phi over those rows (the outer edge node of
 // E_phi, i = i_d1, is not among them).
-__global__ void k_focal_nn(const float *__restrict__ y, int nq, int i_d0, int nrd, int nphi, int nr, float scale,
-                           const double2 *__restrict__ Gr, const double2 *__restrict__ Gp,
-                           const double2 *__restrict__ emph_n, const double2 *__restrict__ emph_h, double2 *S)
+// FP64 arithmetic bounds it, so a (q, b) sum is shared by a cluster of blocks
+// (one warp per row; the radial weight once per row and lane) whose partial
+// sums the first block adds in order: 136 us with one block per sum at
+// 128 x 128 pixels and 6 frequencies.  VEC: y is 16-byte aligned.
+constexpr int FOCAL_SPLIT = 8;
+template <bool VEC>
+__global__ void __cluster_dims__(1, 1, FOCAL_SPLIT) __launch_bounds__(256)
+    k_focal_nn(const float *__restrict__ y, int nq, int i_d0, int nrd, int nphi, int nr, float scale,
+               const double2 *__restrict__ Gr, const double2 *__restrict__ Gp,
+               const double2 *__restrict__ emph_n, const double2 *__restrict__ emph_h, double2 *S)
 {
-    const int q = blockIdx.x, b = blockIdx.y;
+    __shared__ double2 part[FOCAL_SPLIT];
+    const int q = blockIdx.x, b = blockIdx.y, warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int nch = 4 * nq;
+    cooperative_groups::cluster_group cl = cooperative_groups::this_cluster();
+    auto started = cl.barrier_arrive();                      // the first block's shared memory is there
     double2 acc = make_double2(0, 0);
-    for (int t = threadIdx.x; t < nrd * nphi; t += blockDim.x) {
-        const int id = t / nphi, j = t % nphi, i = i_d0 + id;
-        const float *v = y + (((size_t)b * nrd + id) * nphi + j) * nch + q * 4;
-        const double2 er = make_double2((double)v[0] * scale, (double)v[1] * scale);
-        const double2 ep = make_double2((double)v[2] * scale, (double)v[3] * scale);
-        const double2 a = d_cmul(Gr[(size_t)q * nr + i], d_cmul(emph_n[j], er));
-        const double2 c = d_cmul(Gp[(size_t)q * nr + i], d_cmul(emph_h[j], ep));
+    for (int id = blockIdx.z * 8 + warp; id < nrd; id += FOCAL_SPLIT * 8) {
+        double2 sr = make_double2(0, 0), sp = make_double2(0, 0);
+        for (int j = lane; j < nphi; j += 32) {
+            const float *v = y + (((size_t)b * nrd + id) * nphi + j) * nch + q * 4;
+            float4 f;
+            if (VEC) f = __ldg(reinterpret_cast<const float4 *>(v));
+            else f = make_float4(v[0], v[1], v[2], v[3]);
+            const double2 a = d_cmul(emph_n[j], make_double2((double)f.x, (double)f.y));
+            const double2 c = d_cmul(emph_h[j], make_double2((double)f.z, (double)f.w));
+            sr.x += a.x; sr.y += a.y;
+            sp.x += c.x; sp.y += c.y;
+        }
+        const double2 a = d_cmul(Gr[(size_t)q * nr + i_d0 + id], sr), c = d_cmul(Gp[(size_t)q * nr + i_d0 + id], sp);
         acc.x += a.x + c.x;
         acc.y += a.y + c.y;
     }
     acc = block_sum2(acc);
-    if (threadIdx.x == 0) S[(size_t)b * nq + q] = acc;
+    cl.barrier_wait(std::move(started));
+    if (threadIdx.x == 0) *cl.map_shared_rank(&part[cl.block_rank()], 0) = acc;
+    cl.sync();
+    if (cl.block_rank() == 0 && threadIdx.x == 0) {
+        double2 s = make_double2(0, 0);
+        for (int k = 0; k < FOCAL_SPLIT; ++k) {
+            s.x += part[k].x;
+            s.y += part[k].y;
+        }
+        S[(size_t)b * nq + q] = make_double2(s.x * scale, s.y * scale);
+    }
 }
 
 // Transpose: dy = d obj / d y for G = dobj/dRe S + i dobj/dIm S per (b, q):
@@ -656,7 +684,9 @@ void launch_focal_nn(const float *y, int n, int nq, int i_d0, int nrd, int nphi,
                      const double2 *Gr, const double2 *Gp, const double2 *emph_n, const double2 *emph_h, double2 *S,
                      cudaStream_t s)
 {
-    k_focal_nn<<<dim3(nq, n), 256, 0, s>>>(y, nq, i_d0, nrd, nphi, nr, scale, Gr, Gp, emph_n, emph_h, S);
+    const dim3 g(nq, n, FOCAL_SPLIT);
+    if (((uintptr_t)y & 15) == 0) k_focal_nn<true><<<g, 256, 0, s>>>(y, nq, i_d0, nrd, nphi, nr, scale, Gr, Gp, emph_n, emph_h, S);
+    else k_focal_nn<false><<<g, 256, 0, s>>>(y, nq, i_d0, nrd, nphi, nr, scale, Gr, Gp, emph_n, emph_h, S);
 }
 
 void launch_focal_nn_T(const double2 *G, int n, int nq, int i_d0, int nrd, int nphi, int nr, float scale,

@@ -210,46 +210,75 @@ __global__ void k_skip_combine(const uint16_t *gs, const uint16_t *gc, Lev Cc, c
     *reinterpret_cast<uint4 *>(out + pofs(F.rows, c8, pos)) = o;
 }
 
-// column sums of a planar bf16 tensor of `planes` planes over positions < P
-// (channels < nc): partial[block][c]; thread t covers channel t % 8 of rows
-// t / 8, t / 8 + 32, ... of each plane.
-__global__ void k_colsum(const uint16_t *g, long rows, long P, int planes, int nc, float *partial)
+// Column sums of a planar bf16 tensor over positions < P (channels < nc):
+// partial[block][c].  One plane (8 channels) per blockIdx.y; a thread sums
+// whole 16-byte rows, four of them in flight, so the kernel is bound by
+// reading g once.  (One 2-byte channel per thread took 1.39 ms of the 4.9 ms of
+// a 64 x 128 x 128 batch's gradient.)
+__global__ void __launch_bounds__(256) k_colsum(const uint16_t *g, long rows, long P, int nc, float *partial)
 {
-    __shared__ float red[256];
-    const int e = threadIdx.x % 8, r0 = threadIdx.x / 8;
-    for (int c8 = 0; c8 < planes; ++c8) {
-        float acc = 0.f;
-        for (long p = (long)blockIdx.x * 32 + r0; p < P; p += (long)gridDim.x * 32) acc += bf2f(g[pofs(rows, c8, p) + e]);
-        red[threadIdx.x] = acc;
-        __syncthreads();
-        if (threadIdx.x < 8) {
-            float s = 0.f;
-            for (int r = 0; r < 32; ++r) s += red[r * 8 + threadIdx.x];
-            const int c = c8 * 8 + threadIdx.x;
-            if (c < nc) partial[(size_t)blockIdx.x * nc + c] = s;
+    __shared__ float red[8][8];
+    const int c8 = blockIdx.y;
+    const long step = (long)gridDim.x * 256;
+    const uint4 *src = reinterpret_cast<const uint4 *>(g + pofs(rows, c8, 0));
+    float acc[8] = {0, 0, 0, 0, 0, 0, 0, 0};
+    auto add = [&](const uint4 &v) {
+        const uint32_t w[4] = {v.x, v.y, v.z, v.w};
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {
+            acc[2 * e] += __uint_as_float(w[e] << 16);
+            acc[2 * e + 1] += __uint_as_float(w[e] & 0xffff0000u);
         }
-        __syncthreads();
+    };
+    long p = (long)blockIdx.x * 256 + threadIdx.x;
+    for (; p + 3 * step < P; p += 4 * step) {
+        const uint4 a = __ldg(src + p), b = __ldg(src + p + step), c = __ldg(src + p + 2 * step), d = __ldg(src + p + 3 * step);
+        add(a);
+        add(b);
+        add(c);
+        add(d);
+    }
+    for (; p < P; p += step) add(__ldg(src + p));
+#pragma unroll
+    for (int e = 0; e < 8; ++e)
+        for (int o = 16; o > 0; o >>= 1) acc[e] += __shfl_xor_sync(0xffffffffu, acc[e], o);
+    if ((threadIdx.x & 31) == 0)
+#pragma unroll
+        for (int e = 0; e < 8; ++e) red[threadIdx.x >> 5][e] = acc[e];
+    __syncthreads();
+    if (threadIdx.x < 8) {
+        float t = 0.f;
+        for (int w = 0; w < 8; ++w) t += red[w][threadIdx.x];
+        const int c = c8 * 8 + threadIdx.x;
+        if (c < nc) partial[(size_t)blockIdx.x * nc + c] = t;
     }
 }
 
 // Layer gradient from the wgrad partials [splits][ngroups][128][N] and the
-// bias partials [nblk][cout]: grads[w[co][t][ci]], grads[b[co]].
-__global__ void k_layer_grad(const float *wpart, int splits, int ngroups, int ntap_grp, int cin_pad, int N,
-                             const float *bpart, int nblk, int cout, int cin, int taps, float *grad)
+// bias partials [nblk][cout]: grads[w[co][t][ci]], grads[b[co]].  One block per
+// (tap group, row) = (tap, c_in), one more for the bias: lanes along c_out, so
+// the partials are read in whole lines, 256 / N of them at a time.  (Threads
+// along c_in, each walking all splits alone: 20 us a layer, 213 us of the
+// 1.05 ms of a one-sample gradient.)
+__global__ void __launch_bounds__(256) k_layer_grad(const float *wpart, int splits, int ngroups, int ntap_grp, int cin_pad, int N,
+                                                    const float *bpart, int nblk, int cout, int cin, int taps, float *grad)
 {
-    const long i = (long)blockIdx.x * blockDim.x + threadIdx.x;
-    const long nw = (long)cout * taps * cin;
-    if (i < nw) {
-        const int ci = (int)(i % cin), t = (int)((i / cin) % taps), co = (int)(i / ((long)cin * taps));
-        const int g = t / ntap_grp, row = (t % ntap_grp) * cin_pad + ci;
-        float s = 0.f;
-        for (int k = 0; k < splits; ++k) s += wpart[(((size_t)k * ngroups + g) * 128 + row) * N + co];
-        grad[i] = s;
-    } else if (i < nw + cout) {
-        const int co = (int)(i - nw);
-        float s = 0.f;
-        for (int k = 0; k < nblk; ++k) s += bpart[(size_t)k * cout + co];
-        grad[i] = s;
+    __shared__ float red[256];
+    const int co = threadIdx.x % N, part = threadIdx.x / N, parts = 256 / N;
+    const bool bias = blockIdx.x == (unsigned)(ngroups * 128);
+    const int g = blockIdx.x / 128, row = blockIdx.x % 128, t = g * ntap_grp + row / cin_pad, ci = row % cin_pad;
+    if (!bias && (t >= taps || ci >= cin)) return;
+    const float *src = bias ? bpart + co : wpart + ((size_t)g * 128 + row) * N + co;
+    const size_t stride = bias ? (size_t)cout : (size_t)ngroups * 128 * N;
+    const int count = bias ? (co < cout ? nblk : 0) : splits;
+    float s = 0.f;
+#pragma unroll 8
+    for (int k = part; k < count; k += parts) s += __ldg(src + k * stride);
+    red[threadIdx.x] = s;
+    __syncthreads();
+    if (part == 0 && co < cout) {
+        for (int q = 1; q < parts; ++q) s += red[q * N + co];
+        grad[bias ? (long)cout * taps * cin + co : ((long)co * taps + t) * cin + ci] = s;
     }
 }
 
@@ -327,12 +356,18 @@ __global__ void k_mse(const float *y, const float *t, long n, float *dy, float *
     if (threadIdx.x == 0) partial[blockIdx.x] = red[0];
 }
 
-__global__ void k_mse_final(const float *partial, int nblk, long n, float *loss)
+__global__ void __launch_bounds__(256) k_mse_final(const float *partial, int nblk, long n, float *loss)
 {
-    if (threadIdx.x != 0 || blockIdx.x != 0) return;
+    __shared__ double red[256];
     double s = 0.0;
-    for (int b = 0; b < nblk; ++b) s += partial[b];
-    *loss = (float)(s / (double)n);
+    for (int b = threadIdx.x; b < nblk; b += 256) s += partial[b];
+    red[threadIdx.x] = s;
+    __syncthreads();
+    for (int o = 128; o > 0; o >>= 1) {
+        if (threadIdx.x < o) red[threadIdx.x] += red[threadIdx.x + o];
+        __syncthreads();
+    }
+    if (threadIdx.x == 0) *loss = (float)(red[0] / (double)n);
 }
 
 unsigned nblocks(long n, int t = 256) { return (unsigned)((n + t - 1) / t); }
@@ -521,11 +556,12 @@ zda_status layer_grad(zda_nn *net, int li, int n, const uint16_t *x0, const uint
     p.wait_limit = 1 << 22;
     cudaError_t e = launch_wgrad(p, splits, s);
     if (e != cudaSuccess) return nn_fail(ZDA_ERR_CUDA, std::string("wgrad launch: ") + cudaGetErrorString(e));
-    k_colsum<<<net->bpart_blocks, 256, 0, s>>>(g, p.rows, p.P, ldg / 8, l.cout, at<float>(net, net->o.bpart));
-    const long nw = (long)l.cout * p.taps * l.cin + l.cout;
-    k_layer_grad<<<nblocks(nw), 256, 0, s>>>(at<float>(net, net->o.wpart), splits, p.ngroups, p.ntap_grp, l.cin_pad,
-                                             p.N, at<float>(net, net->o.bpart), net->bpart_blocks, l.cout, l.cin,
-                                             p.taps, at<float>(net, net->o.grads) + l.off);
+    // bias partials: blocks of at least 1024 positions per plane, so that small levels leave few of them
+    const int nblk = (int)std::max<long>(1, std::min<long>(net->bpart_blocks, p.P / 1024));
+    k_colsum<<<dim3(nblk, ldg / 8), 256, 0, s>>>(g, p.rows, p.P, l.cout, at<float>(net, net->o.bpart));
+    k_layer_grad<<<p.ngroups * 128 + 1, 256, 0, s>>>(at<float>(net, net->o.wpart), splits, p.ngroups, p.ntap_grp, l.cin_pad,
+                                                     p.N, at<float>(net, net->o.bpart), nblk, l.cout, l.cin, p.taps,
+                                                     at<float>(net, net->o.grads) + l.off);
     net->launches += 3;
     e = cudaGetLastError();
     if (e != cudaSuccess) return nn_fail(ZDA_ERR_CUDA, std::string("gradient reduction: ") + cudaGetErrorString(e));
@@ -830,7 +866,7 @@ zda_status zda_nn_mse(zda_nn *net, const float *y, const float *t, int n, float 
     const long cnt = (long)n * net->d.height * net->d.width * net->d.out_ch;
     const int nb = (int)std::min<long>(1024, nblocks(cnt));
     k_mse<<<nb, 256, 0, s>>>(y, t, cnt, dy, at<float>(net, net->o.mpart));
-    k_mse_final<<<1, 32, 0, s>>>(at<float>(net, net->o.mpart), nb, cnt, loss);
+    k_mse_final<<<1, 256, 0, s>>>(at<float>(net, net->o.mpart), nb, cnt, loss);
     net->launches += 2;
     NN_CUDA(cudaGetLastError());
     return ZDA_OK;
