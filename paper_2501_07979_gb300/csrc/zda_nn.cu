@@ -254,30 +254,51 @@ __global__ void __launch_bounds__(256) k_colsum(const uint16_t *g, long rows, lo
     }
 }
 
-// Layer gradient from the wgrad partials [splits][ngroups][128][N] and the
-// bias partials [nblk][cout]: grads[w[co][t][ci]], grads[b[co]].  One block per
-// (tap group, row) = (tap, c_in), one more for the bias: lanes along c_out, so
-// the partials are read in whole lines, 256 / N of them at a time.  (Threads
-// along c_in, each walking all splits alone: 20 us a layer, 213 us of the
-// 1.05 ms of a one-sample gradient.)
-__global__ void __launch_bounds__(256) k_layer_grad(const float *wpart, int splits, int ngroups, int ntap_grp, int cin_pad, int N,
-                                                    const float *bpart, int nblk, int cout, int cin, int taps, float *grad)
+// Layer gradient from the wgrad partials and the bias partials [nblk][cout]:
+// grads[w[co][t][ci]], grads[b[co]].  A block sums 64 neighbouring values of the
+// partials (a whole 256-byte line of every split) with 16 threads to a value;
+// the last block sums the biases.  Bound by the latency of its few rounds of
+// loads.  (Threads along c_in, each walking all splits alone: 20 us a layer,
+// 213 us of the 1.05 ms of a one-sample gradient.)
+// win = 0: [splits][ngroups][128][N] of k_wgrad_tc; 1: [tensors][splits][6][16][128][4] of k_wgrad_win.
+constexpr int LG_THREADS = 1024, LG_VALUES = 64, LG_PARTS = LG_THREADS / LG_VALUES;
+__global__ void __launch_bounds__(LG_THREADS) k_layer_grad(const float *wpart, int win, int splits, int ngroups, int ntap_grp,
+                                                           int cin_pad, int N, const float *bpart, int nblk, int cout,
+                                                           int cin, int taps, float *grad)
 {
-    __shared__ float red[256];
-    const int co = threadIdx.x % N, part = threadIdx.x / N, parts = 256 / N;
-    const bool bias = blockIdx.x == (unsigned)(ngroups * 128);
-    const int g = blockIdx.x / 128, row = blockIdx.x % 128, t = g * ntap_grp + row / cin_pad, ci = row % cin_pad;
-    if (!bias && (t >= taps || ci >= cin)) return;
-    const float *src = bias ? bpart + co : wpart + ((size_t)g * 128 + row) * N + co;
-    const size_t stride = bias ? (size_t)cout : (size_t)ngroups * 128 * N;
-    const int count = bias ? (co < cout ? nblk : 0) : splits;
+    __shared__ float red[LG_THREADS];
+    const int lane = threadIdx.x % LG_VALUES, part = threadIdx.x / LG_VALUES;
+    const bool bias = blockIdx.x + 1 == gridDim.x;
+    const long v = (long)blockIdx.x * LG_VALUES + lane;      // value of one split's partial (all tensors in turn)
+    const int per = (win ? WW_GROUPS : ngroups) * 128 * N;   // values of a split
+    int co, t, ci;
+    size_t first = (size_t)v;
+    if (win) {
+        const int half = (int)(v / per), w = (int)(v % per), g = w / (128 * 64), row = w / 4 % 128;
+        co = w / 512 % 16 * 4 + w % 4;
+        t = g / 2 * 3 + ((g & 1) ? 2 : row / 64);
+        ci = half * 64 + row % 64;
+        if ((g & 1) && row >= 64) t = taps;                  // the unused second tap
+        first = (size_t)half * splits * per + w;
+    } else {
+        const int row = (int)(v / N) % 128, g = (int)(v / (128 * N));
+        co = (int)(v % N);
+        t = g * ntap_grp + row / cin_pad;
+        ci = row % cin_pad;
+    }
+    if (bias) co = lane;
+    const bool on = co < cout && (bias || (t < taps && ci < cin));
+    const float *src = bias ? bpart + lane : wpart + first;
+    const size_t stride = bias ? (size_t)cout : (size_t)per;
+    const int count = on ? (bias ? nblk : splits) : 0;
     float s = 0.f;
-#pragma unroll 8
-    for (int k = part; k < count; k += parts) s += __ldg(src + k * stride);
+#pragma unroll 10
+    for (int k = part; k < count; k += LG_PARTS) s += __ldg(src + k * stride);
     red[threadIdx.x] = s;
     __syncthreads();
-    if (part == 0 && co < cout) {
-        for (int q = 1; q < parts; ++q) s += red[q * N + co];
+    if (part == 0 && on) {
+#pragma unroll
+        for (int q = 1; q < LG_PARTS; ++q) s += red[q * LG_VALUES + lane];
         grad[bias ? (long)cout * taps * cin + co : ((long)co * taps + t) * cin + ci] = s;
     }
 }
@@ -530,38 +551,67 @@ zda_status layer_grad(zda_nn *net, int li, int n, const uint16_t *x0, const uint
                       cudaStream_t s)
 {
     const Layer &l = net->L[li];
-    WgradParams p{};
-    p.Hp = net->H[l.level] + 2;
-    p.Wp = net->W[l.level] + 2;
-    p.P = (int)pos_count(net, l.level, n);
-    p.taps = l.k * l.k;
-    p.cin_planes = l.cin_pad / 8;
-    p.ntap_grp = 16 / p.cin_planes;
-    p.ngroups = (p.taps + p.ntap_grp - 1) / p.ntap_grp;
-    p.two_inputs = x1 != nullptr;
-    p.N = ldg;
-    p.kt = WG_KT;
-    p.ntiles = (p.P + p.kt - 1) / p.kt;
-    int splits = std::max(1, std::min(p.ntiles, (304 + p.ngroups - 1) / p.ngroups));
-    p.tiles_per_cta = (p.ntiles + splits - 1) / splits;
-    splits = (p.ntiles + p.tiles_per_cta - 1) / p.tiles_per_cta;
-    if ((size_t)splits * p.ngroups * 128 * p.N > net->wpart_floats)
-        return nn_fail(ZDA_ERR_OOM, "weight-gradient partial buffer too small");
-    p.rows = net->rows[l.level];
-    p.x0 = x0;
-    p.x1 = x1;
-    p.dy = g;
-    p.partial = at<float>(net, net->o.wpart);
-    p.err = at<int>(net, net->o.err);
-    p.wait_limit = 1 << 22;
-    cudaError_t e = launch_wgrad(p, splits, s);
+    const long P = pos_count(net, l.level, n), rows = net->rows[l.level];
+    const int Wp = net->W[l.level] + 2, taps = l.k * l.k;
+    // all 3x3 layers but the first have 64 channels per tensor and fit the one-window kernel
+    const bool win = taps == 9 && l.cin_pad % C == 0 && ldg == C && Wp + 1 <= WW_MAX_HALO;
+    int splits, ngroups = 0, ntap_grp = 0, nrow;
+    cudaError_t e;
+    if (win) {
+        WgradWinParams p{};
+        p.P = (int)P;
+        p.Wp = Wp;
+        p.ntiles = (int)((P + WW_TILE - 1) / WW_TILE);
+        const int tensors = x1 ? 2 : 1, ctas = WW_CTAS / tensors;
+        p.tiles_per_cta = std::max(WW_MIN_TILES, (p.ntiles + ctas - 1) / ctas);
+        splits = (p.ntiles + p.tiles_per_cta - 1) / p.tiles_per_cta;
+        nrow = tensors * WW_GROUPS * 128;
+        if ((size_t)splits * nrow * C > net->wpart_floats)
+            return nn_fail(ZDA_ERR_OOM, "weight-gradient partial buffer too small");
+        p.rows = rows;
+        p.x0 = x0;
+        p.x1 = x1;
+        p.dy = g;
+        p.partial = at<float>(net, net->o.wpart);
+        p.err = at<int>(net, net->o.err);
+        p.wait_limit = 1 << 22;
+        e = launch_wgrad_win(p, splits, s);
+    } else {
+        WgradParams p{};
+        p.Hp = net->H[l.level] + 2;
+        p.Wp = Wp;
+        p.P = (int)P;
+        p.taps = taps;
+        p.cin_planes = l.cin_pad / 8;
+        p.ntap_grp = ntap_grp = 16 / p.cin_planes;
+        p.ngroups = ngroups = (p.taps + p.ntap_grp - 1) / p.ntap_grp;
+        p.two_inputs = x1 != nullptr;
+        p.N = ldg;
+        p.kt = WG_KT;
+        p.ntiles = (p.P + p.kt - 1) / p.kt;
+        splits = std::max(1, std::min(p.ntiles, (304 + p.ngroups - 1) / p.ngroups));
+        p.tiles_per_cta = (p.ntiles + splits - 1) / splits;
+        splits = (p.ntiles + p.tiles_per_cta - 1) / p.tiles_per_cta;
+        nrow = ngroups * 128;
+        if ((size_t)splits * nrow * p.N > net->wpart_floats)
+            return nn_fail(ZDA_ERR_OOM, "weight-gradient partial buffer too small");
+        p.rows = rows;
+        p.x0 = x0;
+        p.x1 = x1;
+        p.dy = g;
+        p.partial = at<float>(net, net->o.wpart);
+        p.err = at<int>(net, net->o.err);
+        p.wait_limit = 1 << 22;
+        e = launch_wgrad(p, splits, s);
+    }
     if (e != cudaSuccess) return nn_fail(ZDA_ERR_CUDA, std::string("wgrad launch: ") + cudaGetErrorString(e));
     // bias partials: blocks of at least 1024 positions per plane, so that small levels leave few of them
-    const int nblk = (int)std::max<long>(1, std::min<long>(net->bpart_blocks, p.P / 1024));
-    k_colsum<<<dim3(nblk, ldg / 8), 256, 0, s>>>(g, p.rows, p.P, l.cout, at<float>(net, net->o.bpart));
-    k_layer_grad<<<p.ngroups * 128 + 1, 256, 0, s>>>(at<float>(net, net->o.wpart), splits, p.ngroups, p.ntap_grp, l.cin_pad,
-                                                     p.N, at<float>(net, net->o.bpart), nblk, l.cout, l.cin, p.taps,
-                                                     at<float>(net, net->o.grads) + l.off);
+    const int nblk = (int)std::max<long>(1, std::min<long>(net->bpart_blocks, P / 1024));
+    k_colsum<<<dim3(nblk, ldg / 8), 256, 0, s>>>(g, rows, P, l.cout, at<float>(net, net->o.bpart));
+    k_layer_grad<<<(unsigned)((long)nrow * ldg / LG_VALUES) + 1, LG_THREADS, 0, s>>>(
+        at<float>(net, net->o.wpart), win ? 1 : 0, splits, ngroups, ntap_grp, l.cin_pad, ldg,
+                                          at<float>(net, net->o.bpart), nblk, l.cout, l.cin, taps,
+                                          at<float>(net, net->o.grads) + l.off);
     net->launches += 3;
     e = cudaGetLastError();
     if (e != cudaSuccess) return nn_fail(ZDA_ERR_CUDA, std::string("gradient reduction: ") + cudaGetErrorString(e));
@@ -646,6 +696,7 @@ zda_status zda_nn_create(int device, const zda_nn_desc *d, zda_nn **out)
         const size_t splits = (size_t)std::min<long>((pos_count(net, l.level, B) + 127) / 128, (304 + ng - 1) / ng) + 1;
         wp = std::max(wp, splits * ng * 128 * (size_t)(i == NL - 1 ? 32 : 64));
     }
+    wp = std::max(wp, (size_t)WW_CTAS * WW_GROUPS * 128 * C);        // k_wgrad_win: one partial per block
     net->wpart_floats = wp;
     net->o.wpart = take(wp * 4);
     net->o.bpart = take((size_t)net->bpart_blocks * 64 * 4);

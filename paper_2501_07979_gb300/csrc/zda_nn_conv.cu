@@ -438,6 +438,133 @@ __global__ void __launch_bounds__(WG_THREADS, 1)
     if (warp == 2) tm_dealloc(tmem, ncols);
 }
 
+// Weight gradient of the 64-channel 3x3 layers, every tap from one window.
+//
+// D[(tap, c_in)][c_out] = sum_p X[p + off(tap)][c_in] dY[p][c_out], both operands
+// MN-major, reduction over positions.  A tap is the same window seen from
+// another start row (a plain change of the descriptor's address: rows are 16
+// bytes without swizzle), so a CTA streams X and dY through shared memory once
+// for all nine taps.  The M = 128 rows of an MMA are two taps: the window is
+// kept twice, the second copy one position ahead, and planes 8..15 are that
+// copy's.  Three window rows times (dx = -1, 0 | 1, -) make six accumulators of
+// 64 columns (384 of the 512 TMEM columns; a quarter of the MMAs' rows is not
+// used).  k_wgrad_tc, which loads X once per pair of taps already shifted, reads
+// 5 times the bytes and was bound by them: 2.27 ms of a 64 x 128 x 128 batch's
+// gradient.
+//
+// The window is a ring of nine 64-position chunks; the tile at positions
+// 64 t .. 64 t + 63 reads chunks t - 3 .. t + 3, so two are in flight.  A K step
+// is 16 consecutive rows at any row: the first 16 rows of the ring are copied
+// behind its end too, for the steps that straddle it.
+// Roles (256 threads): warp 0 lane 0 producer, warps 1 and 2 lane 0 issue three
+// accumulators each, warp 3 owns TMEM; all warps store (0..3 the first three
+// accumulators, 4..7 the others).  Waits are bounded.
+__global__ void __launch_bounds__(WW_THREADS, 1) k_wgrad_win(const WgradWinParams p)
+{
+    constexpr int RING = WW_SLOTS * WW_TILE, ROWS = RING + 16;
+    constexpr uint32_t PLANE = ROWS * 16, DYB = 8 * WW_TILE * 16;
+    extern __shared__ __align__(1024) uint8_t smem[];
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const uint32_t raw = su32(smem), base = (raw + 1023u) & ~1023u;
+    const uint32_t sX = base, sDy = sX + 16 * PLANE, sBar = sDy + WW_DY * DYB;
+    const uint32_t xF = sBar, xE = xF + 8 * WW_SLOTS, dF = xE + 8 * WW_SLOTS, dE = dF + 8 * WW_DY, bDone = dE + 8 * WW_DY;
+    const uint32_t sMisc = bDone + 8;
+    uint32_t *tslot = reinterpret_cast<uint32_t *>(smem + (sMisc - raw));
+    volatile int *abort = reinterpret_cast<volatile int *>(smem + (sMisc + 4 - raw));
+    const int split = blockIdx.x, half = blockIdx.y;
+    const int tile0 = split * p.tiles_per_cta, ntile = min(p.ntiles - tile0, p.tiles_per_cta);
+
+    if (threadIdx.x == 0) {
+        for (int s = 0; s < WW_SLOTS; ++s) {
+            mb_init(xF + 8 * s, 1);
+            mb_init(xE + 8 * s, 2);                // one commit per issuer
+        }
+        for (int s = 0; s < WW_DY; ++s) {
+            mb_init(dF + 8 * s, 1);
+            mb_init(dE + 8 * s, 2);
+        }
+        mb_init(bDone, 2);
+        *abort = 0;
+        mb_fence_init();
+    }
+    if (warp == 3) tm_alloc(sMisc, 512);
+    tc_fence_before();
+    __syncthreads();
+    tc_fence_after();
+    const uint32_t tmem = *tslot;
+
+    if (warp == 0 && lane == 0) {
+        const uint16_t *x = half ? p.x1 : p.x0;
+        bool ok = true;
+        for (int c = 0; c < ntile + 6 && ok; ++c) {          // chunk c: positions 64 (tile0 - 3 + c) ..
+            const int s = c % WW_SLOTS;
+            if (c >= WW_SLOTS && !wait_or_abort(xE + 8 * s, (c / WW_SLOTS - 1) & 1, p.wait_limit, abort, p.err, 31)) break;
+            const long pos = (long)WW_TILE * (tile0 - 3 + c);
+            mb_expect_tx(xF + 8 * s, 16 * WW_TILE * 16 + (s == 0 ? 16 * 256 : 0));
+            for (int j = 0; j < 16; ++j) {
+                const uint16_t *src = x + ((size_t)(j & 7) * p.rows + LEAD + pos + (j >> 3)) * 8;
+                bulk_load(sX + j * PLANE + s * (WW_TILE * 16), src, WW_TILE * 16, xF + 8 * s);
+                if (s == 0) bulk_load(sX + j * PLANE + RING * 16, src, 256, xF + 8 * s);
+            }
+            const int i = c - 6;                             // the tile that this chunk completes
+            if (i < 0) continue;
+            const int d = i % WW_DY;
+            if (i >= WW_DY) ok = wait_or_abort(dE + 8 * d, (i / WW_DY - 1) & 1, p.wait_limit, abort, p.err, 32);
+            if (!ok) break;
+            mb_expect_tx(dF + 8 * d, DYB);
+            for (int j = 0; j < 8; ++j)
+                bulk_load(sDy + d * DYB + j * (WW_TILE * 16),
+                          p.dy + ((size_t)j * p.rows + LEAD + (long)WW_TILE * (tile0 + i)) * 8, WW_TILE * 16, dF + 8 * d);
+        }
+    } else if ((warp == 1 || warp == 2) && lane == 0) {
+        const uint32_t idesc = idesc_bf16(128, 64, 1, 1);
+        const int g0 = (warp - 1) * 3;
+        bool ok = true;
+        for (int c = 0; c < 6 && ok; ++c) ok = wait_or_abort(xF + 8 * c, 0, p.wait_limit, abort, p.err, 33);
+        for (int i = 0; i < ntile && ok; ++i) {
+            const int c = i + 6, d = i % WW_DY;
+            ok = wait_or_abort(xF + 8 * (c % WW_SLOTS), (c / WW_SLOTS) & 1, p.wait_limit, abort, p.err, 33) &&
+                 wait_or_abort(dF + 8 * d, (i / WW_DY) & 1, p.wait_limit, abort, p.err, 34);
+            if (!ok) break;
+            tc_fence_after();
+            const uint64_t bd = sdesc(sDy + d * DYB, 128, WW_TILE * 16);
+#pragma unroll
+            for (int g = 0; g < 3; ++g) {
+                const int gg = g0 + g, off = (gg / 2 - 1) * p.Wp + ((gg & 1) ? 1 : -1);
+                int r = (WW_TILE * (i + 3) + off) % RING;
+#pragma unroll
+                for (int ks = 0; ks < WW_TILE / 16; ++ks) {
+                    tc_mma(tmem + gg * 64, sdesc(sX + r * 16, 128, PLANE), bd + (uint64_t)(ks * 16), idesc, (i | ks) != 0);
+                    r += 16;
+                    if (r >= RING) r -= RING;
+                }
+            }
+            tc_commit(xE + 8 * (i % WW_SLOTS));              // chunk i has served its last tile
+            tc_commit(dE + 8 * d);
+        }
+        if (ok) tc_commit(bDone);
+    }
+    __syncwarp();
+    const bool done = wait_or_abort(bDone, 0, p.wait_limit, abort, p.err, 35);
+    tc_fence_after();
+    // partial [..][group][c_out / 4][row][4]: a warp's 16-byte stores are one run
+    const int row = (warp & 3) * 32 + lane, gb = (warp >> 2) * 3;
+    for (int g = gb; g < gb + 3; ++g) {
+        float4 *out = reinterpret_cast<float4 *>(p.partial + (((size_t)half * gridDim.x + split) * WW_GROUPS + g) * 128 * 64);
+        for (int c16 = 0; c16 < 4; ++c16) {
+            float v[16];
+            tm_ld16(tmem + ((uint32_t)((warp & 3) * 32) << 16) + g * 64 + c16 * 16, v);
+            if (!done) continue;
+#pragma unroll
+            for (int i = 0; i < 4; ++i)
+                out[(c16 * 4 + i) * 128 + row] = make_float4(v[4 * i], v[4 * i + 1], v[4 * i + 2], v[4 * i + 3]);
+        }
+    }
+    tc_fence_before();
+    __syncthreads();
+    if (warp == 3) tm_dealloc(tmem, 512);
+}
+
 size_t conv_smem_bytes(const ConvParams &p)
 {
     const size_t upl = p.cg / 8 < 4 ? p.cg / 8 : 4;
@@ -476,6 +603,16 @@ cudaError_t launch_conv(const ConvParams &p, cudaStream_t s)
     const int ntiles = (p.P + p.mt * 128 - 1) / (p.mt * 128);
     const int grid = std::max(1, std::min(ntiles, sms * per_sm));
     k_conv_tc<<<grid, CONV_THREADS, smem, s>>>(p);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_wgrad_win(const WgradWinParams &p, int splits, cudaStream_t s)
+{
+    const size_t smem = (size_t)16 * (WW_SLOTS * WW_TILE + 16) * 16 + WW_DY * 8 * WW_TILE * 16 +
+                        8 * (2 * WW_SLOTS + 2 * WW_DY + 1) + 8 + 1024;
+    cudaError_t e = cudaFuncSetAttribute(k_wgrad_win, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e != cudaSuccess) return e;
+    k_wgrad_win<<<dim3(splits, p.x1 ? 2 : 1), WW_THREADS, smem, s>>>(p);
     return cudaGetLastError();
 }
 

@@ -73,6 +73,25 @@ struct WgradParams {
     int wait_limit;
 };
 
+// Weight gradient of a 3x3 layer with 64 output channels and 64 input channels per tensor, all taps from one
+// window (k_wgrad_win): six accumulators, pair 2 d + e holding taps (dy = d - 1, dx = -1 | 0) for e = 0 and
+// (dy, dx = 1 | nothing) for e = 1, rows [tap of the pair][c_in].
+struct WgradWinParams {
+    int P, Wp;
+    int ntiles;            // ceil(P / WW_TILE)
+    int tiles_per_cta;
+    long rows;
+    const uint16_t *x0, *x1, *dy;  // x1: second tensor of a concatenated input or null
+    float *partial;        // [tensors][splits][6][64 / 4][128][4]
+    int *err;
+    int wait_limit;
+};
+constexpr int WW_TILE = 64, WW_SLOTS = 9, WW_DY = 3, WW_GROUPS = 6;
+constexpr int WW_CTAS = 152;        // blocks at most (the partial buffer is sized for them)
+constexpr int WW_MIN_TILES = 4;     // tiles per block at least: a block's 196 KB of partials cost about 4 tiles' time
+constexpr int WW_THREADS = 256;
+constexpr int WW_MAX_HALO = 3 * WW_TILE - 1;   // Wp + 1 at most: a tile's window is seven chunks
+
 constexpr int CONV_THREADS = 352;   // persistent convolution: producer, 2 MMA and 8 epilogue warps
 constexpr int WG_THREADS = 128;
 constexpr int WG_KT = 128;
@@ -82,6 +101,7 @@ size_t conv_smem_bytes(const ConvParams &p);
 size_t wgrad_smem_bytes(const WgradParams &p);
 cudaError_t launch_conv(const ConvParams &p, cudaStream_t s);
 cudaError_t launch_wgrad(const WgradParams &p, int splits, cudaStream_t s);
+cudaError_t launch_wgrad_win(const WgradWinParams &p, int splits, cudaStream_t s);
 
 }  // namespace nn
 }  // namespace zda

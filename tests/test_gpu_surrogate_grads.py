@@ -1,6 +1,9 @@
 """Weight and bias gradients of the surrogate at the sizes where their kernels can go wrong.
 
-The bias sums and the reduction of the weight gradient's partials depend on the number of positions.  Widths at both ends of the allowed range, one tile and many, ragged last
+The convolution weight gradient (k_wgrad_win) streams 64-position chunks
+through a ring that tiles read at any row, split over at most 152 blocks; the
+bias sums and the reduction of the partials depend on the number of positions
+too.  Widths at both ends of the allowed range, one tile and many, ragged last
 tiles, more tiles than blocks.  On exact-structure networks (one unit weight per
 output channel: all activations and activation gradients exact), so gradients
 differ from the FP64 oracle's by FP32 summation alone: the 1e-5 of
