@@ -42,7 +42,6 @@ constexpr int C = 64;      // network width
 constexpr int NL = 15;     // parameterised layers
 constexpr int LEV = 4;     // resolution levels
 
-__device__ __forceinline__ float bf2f(uint16_t b) { return __uint_as_float((uint32_t)b << 16); }
 __device__ __forceinline__ uint16_t f2bf(float f)
 {
     __nv_bfloat16 h = __float2bfloat16_rn(f);
@@ -54,160 +53,172 @@ __device__ __forceinline__ bool interior(int y, int x, int Hp, int Wp) { return 
 // Planar element offset of (channel plane c8, position pos) in a tensor of `rows` rows per plane.
 __device__ __forceinline__ size_t pofs(long rows, int c8, long pos) { return ((size_t)c8 * rows + LEAD + pos) * 8; }
 
-// x [n][H][W][ic] f32 -> planar bf16, 16 channels (2 planes), positions < Pt (zero border, zero tail)
-__global__ void k_pack_input(const float *x, int n, int H, int W, int ic, long Pt, long rows, uint16_t *out)
-{
-    const long i = (long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= 2 * Pt) return;
-    const int c8 = (int)(i / Pt);
-    const long pos = i % Pt;
-    const int Hp = H + 2, Wp = W + 2;
-    const long P = (long)n * Hp * Wp;
-    const int rem = (int)(pos % (Hp * Wp)), y = rem / Wp, xx = rem % Wp;
-    uint16_t r[8] = {0, 0, 0, 0, 0, 0, 0, 0};
-    if (pos < P && interior(y, xx, Hp, Wp)) {
-        const float *src = x + (((pos / (Hp * Wp)) * H + (y - 1)) * W + (xx - 1)) * ic;
-        for (int e = 0; e < 8; ++e) {
-            const int c = c8 * 8 + e;
-            if (c < ic) r[e] = f2bf(src[c]);
-        }
-    }
-    *reinterpret_cast<uint4 *>(out + pofs(rows, c8, pos)) = *reinterpret_cast<uint4 *>(r);
-}
+// The kernels below run one thread per position of a group of POS_PL planes
+// (blockIdx.y), over the Pt positions of the 256-position tiles (borders and
+// the tail past the last position are written as zeros).  They are bound by
+// memory: a position is taken apart (two 32-bit divisions) once for its planes,
+// whose loads are in flight together.  (One thread per position and plane with
+// 64-bit divisions: 180 us for k_up and 60 for k_pack_input at 256 x 128 x 128
+// positions, 164 for the k_skip_combine of a 64-sample gradient.)
+constexpr int POS_PL = 4;
 
-// [n][H][W][nc] f32 -> planar bf16, 32 channels (4 planes), positions < Pt (zeros elsewhere)
-__global__ void k_pack_grad(const float *dy, int n, int H, int W, int nc, long Pt, long rows, uint16_t *out)
-{
-    const long i = (long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= 4 * Pt) return;
-    const int c8 = (int)(i / Pt);
-    const long pos = i % Pt;
-    const int Hp = H + 2, Wp = W + 2;
-    const long P = (long)n * Hp * Wp;
-    const int rem = (int)(pos % (Hp * Wp)), y = rem / Wp, x = rem % Wp;
-    uint16_t r[8] = {0, 0, 0, 0, 0, 0, 0, 0};
-    if (pos < P && interior(y, x, Hp, Wp)) {
-        const float *src = dy + (((pos / (Hp * Wp)) * H + (y - 1)) * W + (x - 1)) * nc;
-        for (int e = 0; e < 8; ++e) {
-            const int c = c8 * 8 + e;
-            if (c < nc) r[e] = f2bf(src[c]);
-        }
-    }
-    *reinterpret_cast<uint4 *>(out + pofs(rows, c8, pos)) = *reinterpret_cast<uint4 *>(r);
-}
-
-// The position-parallel kernels below run one thread per (plane, position)
-// over Pt positions (the 256-rounded tail is written as zeros), 64 channels.
 struct Lev {
     int n, H, W;        // samples, interior size of this level
-    long rows, Pt;      // rows per plane, positions covered (multiple of 256)
+    long rows;          // rows per plane
 };
 
-__device__ __forceinline__ bool decode(const Lev &L, long pos, long &s, int &y, int &x)
+__device__ __forceinline__ bool decode(int n, int H, int W, int pos, int &s, int &y, int &x)
 {
-    const int Hp = L.H + 2, Wp = L.W + 2;
+    const int Hp = H + 2, Wp = W + 2;
     s = pos / (Hp * Wp);
-    const int rem = (int)(pos % (Hp * Wp));
+    const int rem = pos - s * (Hp * Wp);
     y = rem / Wp;
-    x = rem % Wp;
-    return s < L.n && interior(y, x, Hp, Wp);
+    x = rem - y * Wp;
+    return s < n && interior(y, x, Hp, Wp);
+}
+__device__ __forceinline__ int this_pos() { return (int)(blockIdx.x * blockDim.x + threadIdx.x); }
+__device__ __forceinline__ uint4 row_of(const uint16_t *t, long rows, int c8, long pos)
+{
+    return __ldg(reinterpret_cast<const uint4 *>(t + pofs(rows, c8, pos)));
+}
+__device__ __forceinline__ void set_row(uint16_t *t, long rows, int c8, long pos, const uint4 &v)
+{
+    *reinterpret_cast<uint4 *>(t + pofs(rows, c8, pos)) = v;
+}
+__device__ __forceinline__ void unpack(const uint4 &q, float *v)
+{
+    const uint32_t w[4] = {q.x, q.y, q.z, q.w};
+#pragma unroll
+    for (int e = 0; e < 4; ++e) {
+        v[2 * e] = __uint_as_float(w[e] << 16);
+        v[2 * e + 1] = __uint_as_float(w[e] & 0xffff0000u);
+    }
+}
+__device__ __forceinline__ uint4 packed(const float *v)
+{
+    uint32_t w[4];
+#pragma unroll
+    for (int e = 0; e < 4; ++e) w[e] = (uint32_t)f2bf(v[2 * e]) | (uint32_t)f2bf(v[2 * e + 1]) << 16;
+    return make_uint4(w[0], w[1], w[2], w[3]);
+}
+
+// src [n][H][W][nc] f32 -> planar bf16, `planes` planes (channels >= nc zero)
+__global__ void k_pack_rows(const float *src, int n, int H, int W, int nc, int planes, long rows, uint16_t *out)
+{
+    const int pos = this_pos();
+    int s, y, x;
+    const bool in = decode(n, H, W, pos, s, y, x);
+    src += (((size_t)s * H + (y - 1)) * W + (x - 1)) * nc;
+    for (int c8 = 0; c8 < planes; ++c8) {
+        float v[8];
+#pragma unroll
+        for (int e = 0; e < 8; ++e) v[e] = in && c8 * 8 + e < nc ? __ldg(src + c8 * 8 + e) : 0.f;
+        set_row(out, rows, c8, pos, packed(v));
+    }
 }
 
 // avgpool: coarse interior (i, j) = mean of fine interior (2i .. 2i+1, 2j .. 2j+1)
 __global__ void k_pool(const uint16_t *in, Lev F, uint16_t *out, Lev Cc)
 {
-    const long i = (long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= 8 * Cc.Pt) return;
-    const int c8 = (int)(i / Cc.Pt);
-    const long pos = i % Cc.Pt;
-    long s;
-    int y, x;
-    uint4 o = make_uint4(0, 0, 0, 0);
-    if (decode(Cc, pos, s, y, x)) {
+    const int pos = this_pos(), c0 = blockIdx.y * POS_PL;
+    int s, y, x;
+    const bool on = decode(Cc.n, Cc.H, Cc.W, pos, s, y, x);
+    const long fp = ((long)s * (F.H + 2) + 2 * y - 1) * (F.W + 2) + 2 * x - 1;
+    uint4 q[POS_PL][4];
+#pragma unroll
+    for (int c = 0; c < POS_PL; ++c)
+#pragma unroll
+        for (int a = 0; a < 4; ++a)
+            q[c][a] = on ? row_of(in, F.rows, c0 + c, fp + (a >> 1) * (F.W + 2) + (a & 1)) : make_uint4(0, 0, 0, 0);
+#pragma unroll
+    for (int c = 0; c < POS_PL; ++c) {
         float acc[8] = {0, 0, 0, 0, 0, 0, 0, 0};
-        for (int a = 0; a < 2; ++a)
-            for (int b = 0; b < 2; ++b) {
-                const long fp = (s * (F.H + 2) + 2 * y - 1 + a) * (F.W + 2) + 2 * x - 1 + b;
-                const uint4 q = *reinterpret_cast<const uint4 *>(in + pofs(F.rows, c8, fp));
-                const uint16_t *h = reinterpret_cast<const uint16_t *>(&q);
-                for (int e = 0; e < 8; ++e) acc[e] += bf2f(h[e]);
-            }
-        uint16_t r[8];
-        for (int e = 0; e < 8; ++e) r[e] = f2bf(0.25f * acc[e]);
-        o = *reinterpret_cast<uint4 *>(r);
+#pragma unroll
+        for (int a = 0; a < 4; ++a) {
+            float v[8];
+            unpack(q[c][a], v);
+#pragma unroll
+            for (int e = 0; e < 8; ++e) acc[e] += v[e];
+        }
+#pragma unroll
+        for (int e = 0; e < 8; ++e) acc[e] *= 0.25f;
+        set_row(out, Cc.rows, c0 + c, pos, packed(acc));
     }
-    *reinterpret_cast<uint4 *>(out + pofs(Cc.rows, c8, pos)) = o;
 }
 
 // nearest upsampling: fine interior (i, j) = coarse interior (i / 2, j / 2)
 __global__ void k_up(const uint16_t *in, Lev Cc, uint16_t *out, Lev F)
 {
-    const long i = (long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= 8 * F.Pt) return;
-    const int c8 = (int)(i / F.Pt);
-    const long pos = i % F.Pt;
-    long s;
-    int y, x;
-    uint4 o = make_uint4(0, 0, 0, 0);
-    if (decode(F, pos, s, y, x)) {
-        const long cp = (s * (Cc.H + 2) + (y - 1) / 2 + 1) * (Cc.W + 2) + (x - 1) / 2 + 1;
-        o = *reinterpret_cast<const uint4 *>(in + pofs(Cc.rows, c8, cp));
-    }
-    *reinterpret_cast<uint4 *>(out + pofs(F.rows, c8, pos)) = o;
+    const int pos = this_pos(), c0 = blockIdx.y * POS_PL;
+    int s, y, x;
+    const bool on = decode(F.n, F.H, F.W, pos, s, y, x);
+    const long cp = ((long)s * (Cc.H + 2) + (y - 1) / 2 + 1) * (Cc.W + 2) + (x - 1) / 2 + 1;
+    uint4 q[POS_PL];
+#pragma unroll
+    for (int c = 0; c < POS_PL; ++c) q[c] = on ? row_of(in, Cc.rows, c0 + c, cp) : make_uint4(0, 0, 0, 0);
+#pragma unroll
+    for (int c = 0; c < POS_PL; ++c) set_row(out, F.rows, c0 + c, pos, q[c]);
 }
 
 // transpose of nearest upsampling (sum over each 2x2 block) times the sign
 // mask of the coarse activation: coarse output
 __global__ void k_up_bwd_mask(const uint16_t *g, Lev F, const uint16_t *act, uint16_t *out, Lev Cc)
 {
-    const long i = (long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= 8 * Cc.Pt) return;
-    const int c8 = (int)(i / Cc.Pt);
-    const long pos = i % Cc.Pt;
-    long s;
-    int y, x;
-    uint4 o = make_uint4(0, 0, 0, 0);
-    if (decode(Cc, pos, s, y, x)) {
-        float acc[8] = {0, 0, 0, 0, 0, 0, 0, 0};
-        for (int a = 0; a < 2; ++a)
-            for (int b = 0; b < 2; ++b) {
-                const long fp = (s * (F.H + 2) + 2 * y - 1 + a) * (F.W + 2) + 2 * x - 1 + b;
-                const uint4 q = *reinterpret_cast<const uint4 *>(g + pofs(F.rows, c8, fp));
-                const uint16_t *h = reinterpret_cast<const uint16_t *>(&q);
-                for (int e = 0; e < 8; ++e) acc[e] += bf2f(h[e]);
-            }
-        const uint4 mq = *reinterpret_cast<const uint4 *>(act + pofs(Cc.rows, c8, pos));
-        const uint16_t *m = reinterpret_cast<const uint16_t *>(&mq);
-        uint16_t r[8];
-        for (int e = 0; e < 8; ++e) r[e] = f2bf(bf2f(m[e]) > 0.f ? acc[e] : 0.f);
-        o = *reinterpret_cast<uint4 *>(r);
+    const int pos = this_pos(), c0 = blockIdx.y * POS_PL;
+    int s, y, x;
+    const bool on = decode(Cc.n, Cc.H, Cc.W, pos, s, y, x);
+    const long fp = ((long)s * (F.H + 2) + 2 * y - 1) * (F.W + 2) + 2 * x - 1;
+    uint4 q[POS_PL][4], m[POS_PL];
+#pragma unroll
+    for (int c = 0; c < POS_PL; ++c) {
+#pragma unroll
+        for (int a = 0; a < 4; ++a)
+            q[c][a] = on ? row_of(g, F.rows, c0 + c, fp + (a >> 1) * (F.W + 2) + (a & 1)) : make_uint4(0, 0, 0, 0);
+        m[c] = on ? row_of(act, Cc.rows, c0 + c, pos) : make_uint4(0, 0, 0, 0);
     }
-    *reinterpret_cast<uint4 *>(out + pofs(Cc.rows, c8, pos)) = o;
+#pragma unroll
+    for (int c = 0; c < POS_PL; ++c) {
+        float acc[8] = {0, 0, 0, 0, 0, 0, 0, 0}, mk[8];
+#pragma unroll
+        for (int a = 0; a < 4; ++a) {
+            float v[8];
+            unpack(q[c][a], v);
+#pragma unroll
+            for (int e = 0; e < 8; ++e) acc[e] += v[e];
+        }
+        unpack(m[c], mk);
+#pragma unroll
+        for (int e = 0; e < 8; ++e) acc[e] = mk[e] > 0.f ? acc[e] : 0.f;
+        set_row(out, Cc.rows, c0 + c, pos, packed(acc));
+    }
 }
 
 // skip gradient of level l: mask(act > 0) * (g_skip + transpose of avgpool applied to g_coarse)
 __global__ void k_skip_combine(const uint16_t *gs, const uint16_t *gc, Lev Cc, const uint16_t *act, uint16_t *out,
                                Lev F)
 {
-    const long i = (long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= 8 * F.Pt) return;
-    const int c8 = (int)(i / F.Pt);
-    const long pos = i % F.Pt;
-    long s;
-    int y, x;
-    uint4 o = make_uint4(0, 0, 0, 0);
-    if (decode(F, pos, s, y, x)) {
-        const uint4 a = *reinterpret_cast<const uint4 *>(gs + pofs(F.rows, c8, pos));
-        const long cp = (s * (Cc.H + 2) + (y - 1) / 2 + 1) * (Cc.W + 2) + (x - 1) / 2 + 1;
-        const uint4 b = *reinterpret_cast<const uint4 *>(gc + pofs(Cc.rows, c8, cp));
-        const uint4 mq = *reinterpret_cast<const uint4 *>(act + pofs(F.rows, c8, pos));
-        const uint16_t *ha = reinterpret_cast<const uint16_t *>(&a), *hb = reinterpret_cast<const uint16_t *>(&b),
-                       *m = reinterpret_cast<const uint16_t *>(&mq);
-        uint16_t r[8];
-        for (int e = 0; e < 8; ++e) r[e] = f2bf(bf2f(m[e]) > 0.f ? bf2f(ha[e]) + 0.25f * bf2f(hb[e]) : 0.f);
-        o = *reinterpret_cast<uint4 *>(r);
+    const int pos = this_pos(), c0 = blockIdx.y * POS_PL;
+    int s, y, x;
+    const bool on = decode(F.n, F.H, F.W, pos, s, y, x);
+    const long cp = ((long)s * (Cc.H + 2) + (y - 1) / 2 + 1) * (Cc.W + 2) + (x - 1) / 2 + 1;
+    const uint4 none = make_uint4(0, 0, 0, 0);
+    uint4 a[POS_PL], b[POS_PL], m[POS_PL];
+#pragma unroll
+    for (int c = 0; c < POS_PL; ++c) {
+        a[c] = on ? row_of(gs, F.rows, c0 + c, pos) : none;
+        b[c] = on ? row_of(gc, Cc.rows, c0 + c, cp) : none;
+        m[c] = on ? row_of(act, F.rows, c0 + c, pos) : none;
     }
-    *reinterpret_cast<uint4 *>(out + pofs(F.rows, c8, pos)) = o;
+#pragma unroll
+    for (int c = 0; c < POS_PL; ++c) {
+        float va[8], vb[8], vm[8];
+        unpack(a[c], va);
+        unpack(b[c], vb);
+        unpack(m[c], vm);
+#pragma unroll
+        for (int e = 0; e < 8; ++e) va[e] = vm[e] > 0.f ? va[e] + 0.25f * vb[e] : 0.f;
+        set_row(out, F.rows, c0 + c, pos, packed(va));
+    }
 }
 
 // Column sums of a planar bf16 tensor over positions < P (channels < nc):
@@ -446,7 +457,8 @@ template <class T> T *at(zda_nn *net, size_t off) { return reinterpret_cast<T *>
 
 long pos_count(const zda_nn *net, int lev, int n) { return (long)n * (net->H[lev] + 2) * (net->W[lev] + 2); }
 long pos_tiles(const zda_nn *net, int lev, int n) { return (pos_count(net, lev, n) + 255) / 256 * 256; }
-Lev lev(const zda_nn *net, int l, int n) { return Lev{n, net->H[l], net->W[l], net->rows[l], pos_tiles(net, l, n)}; }
+dim3 pos_grid(const zda_nn *net, int lev, int n) { return dim3(nblocks(pos_tiles(net, lev, n)), 8 / POS_PL); }
+Lev lev(const zda_nn *net, int l, int n) { return Lev{n, net->H[l], net->W[l], net->rows[l]}; }
 
 void build_layers(zda_nn *net)
 {
@@ -803,8 +815,7 @@ zda_status zda_nn_forward(zda_nn *net, const float *x, int n, float *y, void *st
     cudaStream_t s = (cudaStream_t)stream;
     const int H = net->d.height, W = net->d.width;
     uint16_t *x16 = at<uint16_t>(net, net->o.x16);
-    k_pack_input<<<nblocks(2 * pos_tiles(net, 0, n)), 256, 0, s>>>(x, n, H, W, net->d.in_ch, pos_tiles(net, 0, n),
-                                                                  net->rows[0], x16);
+    k_pack_rows<<<nblocks(pos_tiles(net, 0, n)), 256, 0, s>>>(x, n, H, W, net->d.in_ch, 2, net->rows[0], x16);
     net->launches++;
 #define TRY(e)                          \
     do {                                \
@@ -818,8 +829,8 @@ zda_status zda_nn_forward(zda_nn *net, const float *x, int n, float *y, void *st
                  nullptr, C, nullptr, nullptr, s, lf(net, 2 * l, n)));
         TRY(conv(net, l, n, 9, A(net, l, A_ENCA), nullptr, C, C, Wf(net, 2 * l + 1), Bias(net, 2 * l + 1), C, EPI_RELU_BF16,
                  Aw(net, l, A_ENCB), nullptr, C, nullptr, nullptr, s, lf(net, 2 * l + 1, n)));
-        k_pool<<<nblocks(8 * pos_tiles(net, l + 1, n)), 256, 0, s>>>(A(net, l, A_ENCB), lev(net, l, n),
-                                                                    Aw(net, l + 1, A_IN), lev(net, l + 1, n));
+        k_pool<<<pos_grid(net, l + 1, n), 256, 0, s>>>(A(net, l, A_ENCB), lev(net, l, n), Aw(net, l + 1, A_IN),
+                                                       lev(net, l + 1, n));
         net->launches++;
         inp = A(net, l + 1, A_IN);
         cin = C;
@@ -831,8 +842,7 @@ zda_status zda_nn_forward(zda_nn *net, const float *x, int n, float *y, void *st
     const uint16_t *below = A(net, 3, A_ENCB);
     for (int l = 2; l >= 0; --l) {
         const int li = 8 + 2 * (2 - l);
-        k_up<<<nblocks(8 * pos_tiles(net, l, n)), 256, 0, s>>>(below, lev(net, l + 1, n), Aw(net, l, A_UP),
-                                                              lev(net, l, n));
+        k_up<<<pos_grid(net, l, n), 256, 0, s>>>(below, lev(net, l + 1, n), Aw(net, l, A_UP), lev(net, l, n));
         net->launches++;
         TRY(conv(net, l, n, 9, A(net, l, A_UP), A(net, l, A_ENCB), C, C, Wf(net, li), Bias(net, li), C, EPI_RELU_BF16,
                  Aw(net, l, A_DECA), nullptr, C, nullptr, nullptr, s, lf(net, li, n)));
@@ -856,8 +866,7 @@ zda_status zda_nn_backward(zda_nn *net, const float *dy, float *dx, void *stream
     cudaStream_t s = (cudaStream_t)stream;
     const int n = net->n_fwd, H = net->d.height, W = net->d.width;
     uint16_t *gy = at<uint16_t>(net, net->o.gy);
-    k_pack_grad<<<nblocks(4 * pos_tiles(net, 0, n)), 256, 0, s>>>(dy, n, H, W, net->d.out_ch, pos_tiles(net, 0, n),
-                                                                 net->rows[0], gy);
+    k_pack_rows<<<nblocks(pos_tiles(net, 0, n)), 256, 0, s>>>(dy, n, H, W, net->d.out_ch, 4, net->rows[0], gy);
     net->launches++;
     // head
     TRY(layer_grad(net, 14, n, A(net, 0, A_DECB), nullptr, gy, 32, s));
@@ -873,8 +882,8 @@ zda_status zda_nn_backward(zda_nn *net, const float *dy, float *dx, void *stream
         TRY(conv(net, l, n, 9, Gb(net, l, G_A), nullptr, C, 2 * C, Wd(net, li), nullptr, 0, EPI_GRAD_BF16,
                  Gb(net, l, G_U), Gb(net, l, G_S), C, nullptr, nullptr, s));
         const uint16_t *below = l == 2 ? A(net, 3, A_ENCB) : A(net, l + 1, A_DECB);
-        k_up_bwd_mask<<<nblocks(8 * pos_tiles(net, l + 1, n)), 256, 0, s>>>(Gb(net, l, G_U), lev(net, l, n), below,
-                                                                           Gb(net, l + 1, G_B), lev(net, l + 1, n));
+        k_up_bwd_mask<<<pos_grid(net, l + 1, n), 256, 0, s>>>(Gb(net, l, G_U), lev(net, l, n), below,
+                                                              Gb(net, l + 1, G_B), lev(net, l + 1, n));
         net->launches++;
     }
     // bottleneck (level 3: A_ENCA = bot_a, A_ENCB = bot_b)
@@ -886,9 +895,8 @@ zda_status zda_nn_backward(zda_nn *net, const float *dy, float *dx, void *stream
              nullptr, C, nullptr, nullptr, s));
     // encoder, coarse to fine: G_U of level l + 1 holds the gradient of in_{l+1}
     for (int l = 2; l >= 0; --l) {
-        k_skip_combine<<<nblocks(8 * pos_tiles(net, l, n)), 256, 0, s>>>(Gb(net, l, G_S), Gb(net, l + 1, G_U),
-                                                                        lev(net, l + 1, n), A(net, l, A_ENCB),
-                                                                        Gb(net, l, G_B), lev(net, l, n));
+        k_skip_combine<<<pos_grid(net, l, n), 256, 0, s>>>(Gb(net, l, G_S), Gb(net, l + 1, G_U), lev(net, l + 1, n),
+                                                           A(net, l, A_ENCB), Gb(net, l, G_B), lev(net, l, n));
         net->launches++;
         TRY(layer_grad(net, 2 * l + 1, n, A(net, l, A_ENCA), nullptr, Gb(net, l, G_B), C, s));
         TRY(conv(net, l, n, 9, Gb(net, l, G_B), nullptr, C, C, Wd(net, 2 * l + 1), nullptr, 0, EPI_GRAD_BF16,
