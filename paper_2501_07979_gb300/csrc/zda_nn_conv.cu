@@ -16,10 +16,12 @@
 //               reduction over positions; M = 128 rows hold 128 / c_in taps'
 //               shifted copies of the input, each copied pre-shifted.
 //
-// Roles of k_conv_tc (352 threads): warp 0 lane 0 = producer, warps 1 and 10
+// Roles of k_conv_tc (608 threads): warp 0 lane 0 = producer, warps 1 and 10
 // lane 0 = MMA issuers (M tile 0 / 1 of each tile, warp 1 also allocates
-// TMEM), warps 2..9 = epilogue (warp w reads TMEM lanes 32 (w mod 4) ..).  Every mbarrier wait is bounded; a timeout sets
-// the error word and the CTA skips its stores, frees TMEM and exits.
+// TMEM), warps 2..9 and 11..18 = epilogue (warp w reads TMEM lanes 32 (w mod
+// 4) .., four warps share the 16-channel chunks).  Every mbarrier wait is
+// bounded; a timeout sets the error word and the CTA skips its stores, frees
+// TMEM and exits.
 #include <cuda_bf16.h>
 
 #include <algorithm>
@@ -29,8 +31,6 @@
 
 namespace zda {
 namespace nn {
-
-static __device__ __forceinline__ bool bf16_pos(uint16_t b) { return !(b & 0x8000u) && b != 0; }
 
 static __device__ __forceinline__ uint32_t pack_bf16(float a, float b)
 {
@@ -51,59 +51,80 @@ static __device__ __forceinline__ bool wait_or_abort(uint32_t bar, uint32_t pari
     return false;
 }
 
-// Epilogue of one 16-channel chunk (channels cc .. cc + 15) of one position.
-__device__ __forceinline__ void epilogue_chunk(const ConvParams &p, float *v, int cc, int pos, bool valid, bool inner,
-                                               const float *bias)
+// Two sums at once (each rounded as a single one).
+static __device__ __forceinline__ float2 add2(float2 a, float2 b)
 {
-    if (p.epi == EPI_F32 || p.epi == EPI_GRAD_F32) {
-        // straight into the caller's [n][H][W][out_ld] tensor (interior positions only)
-        if (!inner || cc >= p.out_ld) return;
-        const int HW = p.Hp * p.Wp, rem = pos % HW, y = rem / p.Wp, x = rem % p.Wp;
-        const size_t pix = ((size_t)(pos / HW) * (p.Hp - 2) + (y - 1)) * (p.Wp - 2) + (x - 1);
-        float *o = static_cast<float *>(p.out0) + pix * p.out_ld + cc;
-        const int nc = p.out_ld - cc < 16 ? p.out_ld - cc : 16;
+    unsigned long long r;
+    asm("add.rn.f32x2 %0, %1, %2;"
+        : "=l"(r)
+        : "l"(*reinterpret_cast<unsigned long long *>(&a)), "l"(*reinterpret_cast<unsigned long long *>(&b)));
+    return *reinterpret_cast<float2 *>(&r);
+}
+
+// Epilogue of one 16-channel chunk (channels cc .. cc + 15) of one position,
+// f32: straight into the caller's [n][H][W][out_ld] tensor (interior positions only).
+__device__ __forceinline__ void store_f32(const ConvParams &p, const float *v, int cc, int pos, int y, int x, bool inner,
+                                          const float2 *bias)
+{
+    if (!inner || cc >= p.out_ld) return;
+    const size_t pix = ((size_t)(pos / (p.Hp * p.Wp)) * (p.Hp - 2) + (y - 1)) * (p.Wp - 2) + (x - 1);
+    float *o = static_cast<float *>(p.out0) + pix * p.out_ld + cc;
+    const int nc = p.out_ld - cc < 16 ? p.out_ld - cc : 16;
+    float w[16];
 #pragma unroll
-        for (int i = 0; i < 16; ++i) v[i] += bias[i];
-        if ((p.out_ld & 3) == 0) {
-            float4 *o4 = reinterpret_cast<float4 *>(o);
+    for (int i = 0; i < 8; ++i) *reinterpret_cast<float2 *>(w + 2 * i) = add2(make_float2(v[2 * i], v[2 * i + 1]), bias[i]);
+    if ((p.out_ld & 3) == 0) {
+        float4 *o4 = reinterpret_cast<float4 *>(o);
 #pragma unroll
-            for (int i = 0; i < 4; ++i)
-                if (4 * i < nc) o4[i] = make_float4(v[4 * i], v[4 * i + 1], v[4 * i + 2], v[4 * i + 3]);
-        } else {
+        for (int i = 0; i < 4; ++i)
+            if (4 * i < nc) o4[i] = make_float4(w[4 * i], w[4 * i + 1], w[4 * i + 2], w[4 * i + 3]);
+    } else {
 #pragma unroll
-            for (int i = 0; i < 16; ++i)
-                if (i < nc) o[i] = v[i];
-        }
-        return;
+        for (int i = 0; i < 16; ++i)
+            if (i < nc) o[i] = w[i];
     }
+}
+
+// The same, bf16 planes (border positions and those past P are zero).  ReLU
+// after rounding is ReLU before it; m0, m1: the sign mask's rows of both planes.
+__device__ __forceinline__ void store_bf16(const ConvParams &p, const float *v, int cc, int pos, bool inner,
+                                           const float2 *bias, const uint4 &m0, const uint4 &m1)
+{
     const int half = cc >= p.out_ld ? 1 : 0;
     const int c = cc - half * p.out_ld;           // channel within the output tensor
+    uint32_t w[8];
     if (p.epi == EPI_RELU_BF16) {
 #pragma unroll
-        for (int i = 0; i < 16; ++i) v[i] = inner ? fmaxf(v[i] + bias[i], 0.f) : 0.f;
-    } else {   // EPI_GRAD_BF16
-        const uint16_t *mk = half ? p.mask1 : p.mask0;
-        if (mk && inner) {
-            const uint4 m0 = __ldg(reinterpret_cast<const uint4 *>(mk + ((size_t)(c / 8) * p.rows + LEAD + pos) * 8));
-            const uint4 m1 = __ldg(reinterpret_cast<const uint4 *>(mk + ((size_t)(c / 8 + 1) * p.rows + LEAD + pos) * 8));
-            const uint16_t *h0 = reinterpret_cast<const uint16_t *>(&m0);
-            const uint16_t *h1 = reinterpret_cast<const uint16_t *>(&m1);
-#pragma unroll
-            for (int i = 0; i < 8; ++i) {
-                if (!bf16_pos(h0[i])) v[i] = 0.f;
-                if (!bf16_pos(h1[i])) v[8 + i] = 0.f;
-            }
+        for (int i = 0; i < 8; ++i) {
+            const float2 s = add2(make_float2(v[2 * i], v[2 * i + 1]), bias[i]);
+            const __nv_bfloat162 h = __hmax2(__floats2bfloat162_rn(s.x, s.y), __floats2bfloat162_rn(0.f, 0.f));
+            w[i] = *reinterpret_cast<const uint32_t *>(&h);
         }
-        if (!inner) {
+    } else {   // EPI_GRAD_BF16: keep where the activation was positive
+        const uint32_t m[8] = {m0.x, m0.y, m0.z, m0.w, m1.x, m1.y, m1.z, m1.w};
 #pragma unroll
-            for (int i = 0; i < 16; ++i) v[i] = 0.f;
-        }
+        for (int i = 0; i < 8; ++i) w[i] = pack_bf16(v[2 * i], v[2 * i + 1]) & __vcmpgts2(m[i], 0u);
     }
-    uint16_t *ob = static_cast<uint16_t *>(half ? p.out1 : p.out0);
-    *reinterpret_cast<uint4 *>(ob + ((size_t)(c / 8) * p.rows + LEAD + pos) * 8) =
-        make_uint4(pack_bf16(v[0], v[1]), pack_bf16(v[2], v[3]), pack_bf16(v[4], v[5]), pack_bf16(v[6], v[7]));
-    *reinterpret_cast<uint4 *>(ob + ((size_t)(c / 8 + 1) * p.rows + LEAD + pos) * 8) =
-        make_uint4(pack_bf16(v[8], v[9]), pack_bf16(v[10], v[11]), pack_bf16(v[12], v[13]), pack_bf16(v[14], v[15]));
+    if (!inner) {
+#pragma unroll
+        for (int i = 0; i < 8; ++i) w[i] = 0u;
+    }
+    uint16_t *ob = static_cast<uint16_t *>(half ? p.out1 : p.out0) + ((size_t)(c / 8) * p.rows + LEAD + pos) * 8;
+    *reinterpret_cast<uint4 *>(ob) = make_uint4(w[0], w[1], w[2], w[3]);
+    *reinterpret_cast<uint4 *>(ob + (size_t)p.rows * 8) = make_uint4(w[4], w[5], w[6], w[7]);
+}
+
+// Mask rows of a chunk (all ones where the gradient is not masked).
+__device__ __forceinline__ void load_mask(const ConvParams &p, int cc, int pos, bool inner, uint4 &m0, uint4 &m1)
+{
+    m0 = m1 = make_uint4(0x00010001u, 0x00010001u, 0x00010001u, 0x00010001u);
+    if (p.epi != EPI_GRAD_BF16 || !inner) return;
+    const int half = cc >= p.out_ld ? 1 : 0, c = cc - half * p.out_ld;
+    const uint16_t *mk = half ? p.mask1 : p.mask0;
+    if (!mk) return;
+    mk += ((size_t)(c / 8) * p.rows + LEAD + pos) * 8;
+    m0 = __ldg(reinterpret_cast<const uint4 *>(mk));
+    m1 = __ldg(reinterpret_cast<const uint4 *>(mk + (size_t)p.rows * 8));
 }
 
 // The MMAs of one tap for M tile m0 of the tile: NKS K-steps of 16 channels each.
@@ -146,9 +167,12 @@ __device__ __forceinline__ void mb_arrive(uint32_t bar)
 // weight blocks are either loaded once per CTA (resident: every layer whose
 // weights fit beside the two windows) or streamed per tap through a ring
 // (the concatenating layers); warp 1 (one lane) issues the MMAs
-// into one of two TMEM accumulators (2 x mt x N columns); warps 2..9 drain
-// the other accumulator (warp w reads lane quarter w mod 4, column half
-// (w - 2) / 4) while the next tile's MMAs run.
+// into one of two TMEM accumulators (2 x mt x N columns); sixteen
+// warps drain the other accumulator while the next tile's MMAs run.  With
+// eight, whose instructions ran at a sixth of a warp's issue rate, a tile's
+// epilogue took 1.6 us and bounded the layers of few MMAs and those that load a
+// mask, which is now loaded before the wait (64 x 128 x 128 positions: first
+// layer 51 -> 43 us, all 30 convolutions of a gradient 1472 -> 1254 us).
 __global__ void __launch_bounds__(CONV_THREADS, 1)
     k_conv_tc(const ConvParams p)
 {
@@ -178,7 +202,7 @@ __global__ void __launch_bounds__(CONV_THREADS, 1)
             mb_init(winFull + 8 * s, 1);
             mb_init(winEmpty + 8 * s, 2);          // one commit per MMA warp
             mb_init(accFull + 8 * s, 2);
-            mb_init(accEmpty + 8 * s, 8);          // one arrival per epilogue warp
+            mb_init(accEmpty + 8 * s, CONV_EPI_WARPS);
         }
         for (int s = 0; s < p.slots; ++s) {
             mb_init(wFull + 8 * s, 1);
@@ -296,44 +320,67 @@ __global__ void __launch_bounds__(CONV_THREADS, 1)
             }
         }
     } else {
-        // ---------------- epilogue (warps 2..9)
-        const int q = warp & 3, h = (warp - 2) >> 2;
+        // ---------------- epilogue: warp quarter q's TMEM lanes, 16-channel chunks h, h + 4, ... of both M tiles
+        const int q = warp & 3, h = (warp < 10 ? warp - 2 : warp - 3) >> 2;
         const int HW = p.Hp * p.Wp, nchunk = p.N / 16;
-        // this warp's chunks: c16 = h, h + 2, h + 4, h + 6 (those < nchunk); biases in registers
-        float bias_r[2][16];
+        const int step = (int)((long)gridDim.x * tile_pos % HW), step128 = 128 % HW;
+        const float inv_wp = 1.f / (float)p.Wp;
+        float2 bias[8];                                // of chunk h (layers with biases have N <= 64)
 #pragma unroll
-        for (int j = 0; j < 2; ++j)
-#pragma unroll
-            for (int i = 0; i < 16; ++i) {
-                const int c = (h + 2 * j) * 16 + i;
-                bias_r[j][i] = (p.bias && c < p.nbias) ? __ldg(p.bias + c) : 0.f;
-            }
+        for (int i = 0; i < 16; ++i) {
+            const int c = h * 16 + i;
+            reinterpret_cast<float *>(bias)[i] = (p.bias && c < p.nbias) ? __ldg(p.bias + c) : 0.f;
+        }
+        int rem0 = (int)(((long)blockIdx.x * tile_pos + q * 32 + lane) % HW);
         for (int t = 0; t < my_tiles; ++t) {
             const int b = t & 1, kb = t >> 1;
+            const int p0 = ((int)blockIdx.x + t * (int)gridDim.x) * tile_pos;
+            // both M tiles' positions: the row by a product (x + 1/2 is at least 1/2 off a multiple of Wp <= 178,
+            // x < 1026 x 178, so rounding cannot reach the next row)
+            int pos[2], y[2], x[2];
+            bool inner[2];
+            uint4 mk[2][2];
+            int rem = rem0;
+#pragma unroll
+            for (int m = 0; m < 2; ++m) {
+                pos[m] = p0 + m * 128 + q * 32 + lane;
+                y[m] = (int)(((float)rem + 0.5f) * inv_wp);
+                x[m] = rem - y[m] * p.Wp;
+                inner[m] = pos[m] < p.P && y[m] > 0 && y[m] < p.Hp - 1 && x[m] > 0 && x[m] < p.Wp - 1;
+                if (h < nchunk) load_mask(p, h * 16, pos[m], inner[m], mk[m][0], mk[m][1]);
+                rem += step128;
+                rem -= rem >= HW ? HW : 0;
+            }
+            rem0 += step;
+            rem0 -= rem0 >= HW ? HW : 0;
             bool ok = true;
             if (lane == 0) ok = wait_or_abort(accFull + 8 * b, kb & 1, p.wait_limit, abort, p.err, 16);
             ok = __shfl_sync(0xffffffffu, ok ? 1 : 0, 0) != 0;
             if (!ok) break;
             tc_fence_after();
-            const int p0 = ((int)blockIdx.x + t * (int)gridDim.x) * tile_pos;
-            for (int m = 0; m < p.mt; ++m) {
-                const int pos = p0 + m * 128 + q * 32 + lane;
-                const bool valid = pos < p.P;             // rows up to the tile end exist (zeroed past P)
-                const int rem = pos % HW, y = rem / p.Wp, x = rem % p.Wp;
-                const bool inner = valid && y > 0 && y < p.Hp - 1 && x > 0 && x < p.Wp - 1;
-                const uint32_t trow = tmem + ((uint32_t)(q * 32) << 16) + b * acc_cols + m * p.N;
-                for (int c16 = h; c16 < nchunk; c16 += 4) {
-                    float va[16], vb[16];
-                    const bool two = c16 + 2 < nchunk;
-                    if (two) tm_ld16x2(trow + c16 * 16, trow + (c16 + 2) * 16, va, vb);
-                    else tm_ld16(trow + c16 * 16, va);
-                    epilogue_chunk(p, va, c16 * 16, pos, valid, inner, bias_r[0]);   // biases only when N <= 64
-                    if (two) epilogue_chunk(p, vb, (c16 + 2) * 16, pos, valid, inner, bias_r[1]);
+            const uint32_t trow = tmem + ((uint32_t)(q * 32) << 16) + b * acc_cols;
+            for (int c16 = h; c16 < nchunk; c16 += 4) {
+                float v[2][16];
+                tm_ld16x2(trow + c16 * 16, trow + p.N + c16 * 16, v[0], v[1]);
+                if (c16 + 4 >= nchunk) {               // the accumulator is free once the last values are out
+                    tc_fence_before();
+                    __syncwarp();
+                    if (lane == 0) mb_arrive(accEmpty + 8 * b);
+                }
+#pragma unroll
+                for (int m = 0; m < 2; ++m) {
+                    if (p.epi == EPI_F32 || p.epi == EPI_GRAD_F32) {
+                        store_f32(p, v[m], c16 * 16, pos[m], y[m], x[m], inner[m], bias);
+                    } else {
+                        if (c16 != h) load_mask(p, c16 * 16, pos[m], inner[m], mk[m][0], mk[m][1]);
+                        store_bf16(p, v[m], c16 * 16, pos[m], inner[m], bias, mk[m][0], mk[m][1]);
+                    }
                 }
             }
-            tc_fence_before();
-            __syncwarp();
-            if (lane == 0) mb_arrive(accEmpty + 8 * b);
+            if (h >= nchunk) {                         // no chunk for this warp
+                __syncwarp();
+                if (lane == 0) mb_arrive(accEmpty + 8 * b);
+            }
         }
     }
     __syncwarp();

@@ -92,7 +92,8 @@ constexpr int WW_MIN_TILES = 4;     // tiles per block at least: a block's 196 K
 constexpr int WW_THREADS = 256;
 constexpr int WW_MAX_HALO = 3 * WW_TILE - 1;   // Wp + 1 at most: a tile's window is seven chunks
 
-constexpr int CONV_THREADS = 352;   // persistent convolution: producer, 2 MMA and 8 epilogue warps
+constexpr int CONV_EPI_WARPS = 16;
+constexpr int CONV_THREADS = 32 * (3 + CONV_EPI_WARPS);   // persistent convolution: producer, 2 MMA and the epilogue warps
 constexpr int WG_THREADS = 128;
 constexpr int WG_KT = 128;
 constexpr int WG_STAGES = 2;
