@@ -518,6 +518,7 @@ zda_status conv(zda_nn *net, int lv, int n, int taps, const uint16_t *in0, const
     const size_t upl = std::min(cg / 8, 4);                    // window planes per unit (32 channels)
     const size_t win2 = 2 * upl * p.plane, wslot = (size_t)N * cg * 2, uslot = (size_t)N * upl * 16;
     p.resident = win2 + (size_t)p.ngroups * taps * wslot <= budget ? 1 : 0;
+    p.stages = 2;
     p.slots = p.resident ? 1 : (int)std::max<size_t>(2, std::min<size_t>(8, (budget - win2) / uslot));
     uint32_t nc = 32;
     while (nc < (uint32_t)(2 * p.mt * N)) nc <<= 1;   // two accumulators (double buffering)

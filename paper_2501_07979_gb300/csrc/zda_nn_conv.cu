@@ -177,17 +177,18 @@ __global__ void __launch_bounds__(CONV_THREADS, 1)
     k_conv_tc(const ConvParams p)
 {
     extern __shared__ __align__(1024) uint8_t smem[];
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int warp = warp_index(), lane = threadIdx.x & 31;
     const uint32_t raw = su32(smem), base = (raw + 1023u) & ~1023u;   // copy destinations: 1024-aligned
     // a unit = up to 4 planes (32 channels) of one input group; window stages hold one unit
     const int upl = p.cg / 8 < 4 ? p.cg / 8 : 4, uh = (p.cg / 8) / upl, nunits = p.ngroups * uh;
     const uint32_t win_bytes = (uint32_t)upl * p.plane;
     const uint32_t wslot = (uint32_t)p.N * p.cg * 2;              // one (group, tap) weight block
     const uint32_t uslot = (uint32_t)p.N * upl * 16;              // its share for one unit (streamed ring)
-    const uint32_t sWin = base, sW = base + 2 * win_bytes;
+    const int ns = p.stages;
+    const uint32_t sWin = base, sW = base + ns * win_bytes;
     const uint32_t sBar = sW + (p.resident ? p.ngroups * p.taps * wslot : p.slots * uslot);
-    const uint32_t winFull = sBar, winEmpty = sBar + 16, accFull = sBar + 32, accEmpty = sBar + 48;
-    const uint32_t wFull = sBar + 64, wEmpty = wFull + 8 * p.slots;
+    const uint32_t winFull = sBar, winEmpty = winFull + 8 * ns, accFull = winEmpty + 8 * ns, accEmpty = accFull + 16;
+    const uint32_t wFull = accEmpty + 16, wEmpty = wFull + 8 * p.slots;
     const uint32_t sMisc = wEmpty + 8 * p.slots;
     uint32_t *tslot = reinterpret_cast<uint32_t *>(smem + (sMisc - raw));
     volatile int *abort = reinterpret_cast<volatile int *>(smem + (sMisc + 4 - raw));
@@ -198,9 +199,11 @@ __global__ void __launch_bounds__(CONV_THREADS, 1)
     const uint32_t acc_cols = (uint32_t)(p.mt * p.N);
 
     if (threadIdx.x == 0) {
-        for (int s = 0; s < 2; ++s) {
+        for (int s = 0; s < ns; ++s) {
             mb_init(winFull + 8 * s, 1);
             mb_init(winEmpty + 8 * s, 2);          // one commit per MMA warp
+        }
+        for (int s = 0; s < 2; ++s) {
             mb_init(accFull + 8 * s, 2);
             mb_init(accEmpty + 8 * s, CONV_EPI_WARPS);
         }
@@ -215,10 +218,10 @@ __global__ void __launch_bounds__(CONV_THREADS, 1)
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
-    const uint32_t tmem = *tslot;
+    const uint32_t tmem = __shfl_sync(0xffffffffu, *tslot, 0);
 
     if (warp == 0) {
-        if (lane == 0) {
+        if (elect_one()) {
             // ---------------- producer
             int u = 0, it = 0;
             bool ok = true;
@@ -231,7 +234,7 @@ __global__ void __launch_bounds__(CONV_THREADS, 1)
                 const int p0 = ((int)blockIdx.x + t * (int)gridDim.x) * tile_pos;
                 for (int uu = 0; uu < nunits && ok; ++uu, ++u) {
                     const int g = uu / uh, hf = uu % uh;
-                    const int s = u & 1, k = u >> 1;
+                    const int s = u % ns, k = u / ns;
                     if (k > 0 && !wait_or_abort(winEmpty + 8 * s, (k - 1) & 1, p.wait_limit, abort, p.err, 11)) {
                         ok = false;
                         break;
@@ -257,7 +260,7 @@ __global__ void __launch_bounds__(CONV_THREADS, 1)
             }
         }
     } else if (warp == 1 || warp == 10) {
-        if (lane == 0) {
+        if (elect_one()) {
             // ---------------- MMA issuers: warp 1 issues M tile 0, warp 10 M tile 1 (separate accumulators)
             const int m0 = warp == 1 ? 0 : 1;
             const uint32_t idesc = idesc_bf16(128, p.N, 0, 0);
@@ -278,7 +281,7 @@ __global__ void __launch_bounds__(CONV_THREADS, 1)
                 const uint32_t d0 = tmem + b * acc_cols;
                 for (int uu = 0; uu < nunits && ok; ++uu, ++u) {
                     const int g = uu / uh, hf = uu % uh;
-                    const int s = u & 1, k = u >> 1;
+                    const int s = u % ns, k = u / ns;
                     if (!wait_or_abort(winFull + 8 * s, k & 1, p.wait_limit, abort, p.err, 14)) {
                         ok = false;
                         break;
@@ -393,7 +396,7 @@ __global__ void __launch_bounds__(WG_THREADS, 1)
     k_wgrad_tc(const WgradParams p)
 {
     extern __shared__ __align__(1024) uint8_t smem[];
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int warp = warp_index(), lane = threadIdx.x & 31;
     const uint32_t raw = su32(smem), base = (raw + 1023u) & ~1023u;
     const uint32_t planeb = (uint32_t)p.kt * 16;
     const uint32_t a_bytes = 16 * planeb, b_bytes = (uint32_t)(p.N / 8) * planeb;
@@ -420,9 +423,9 @@ __global__ void __launch_bounds__(WG_THREADS, 1)
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
-    const uint32_t tmem = *tslot;
+    const uint32_t tmem = __shfl_sync(0xffffffffu, *tslot, 0);
 
-    if (warp == 0 && lane == 0) {
+    if (warp == 0 && elect_one()) {
         for (int i = 0; i < ntile; ++i) {
             const int s = i % WG_STAGES, u = i / WG_STAGES;
             if (u > 0 && !mb_wait(barE + 8 * s, (u - 1) & 1, p.wait_limit, p.err, 21)) break;
@@ -444,7 +447,7 @@ __global__ void __launch_bounds__(WG_THREADS, 1)
             for (int c = 0; c < p.N / 8; ++c)
                 bulk_load(sb + c * planeb, p.dy + ((size_t)c * p.rows + LEAD + y) * 8, planeb, barF + 8 * s);
         }
-    } else if (warp == 1 && lane == 0) {
+    } else if (warp == 1 && elect_one()) {
         const uint32_t idesc = idesc_bf16(128, p.N, 1, 1);
         bool ok = true;
         for (int i = 0; i < ntile; ++i) {
@@ -511,7 +514,7 @@ __global__ void __launch_bounds__(WW_THREADS, 1) k_wgrad_win(const WgradWinParam
     constexpr int RING = WW_SLOTS * WW_TILE, ROWS = RING + 16;
     constexpr uint32_t PLANE = ROWS * 16, DYB = 8 * WW_TILE * 16;
     extern __shared__ __align__(1024) uint8_t smem[];
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int warp = warp_index(), lane = threadIdx.x & 31;
     const uint32_t raw = su32(smem), base = (raw + 1023u) & ~1023u;
     const uint32_t sX = base, sDy = sX + 16 * PLANE, sBar = sDy + WW_DY * DYB;
     const uint32_t xF = sBar, xE = xF + 8 * WW_SLOTS, dF = xE + 8 * WW_SLOTS, dE = dF + 8 * WW_DY, bDone = dE + 8 * WW_DY;
@@ -538,9 +541,9 @@ __global__ void __launch_bounds__(WW_THREADS, 1) k_wgrad_win(const WgradWinParam
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
-    const uint32_t tmem = *tslot;
+    const uint32_t tmem = __shfl_sync(0xffffffffu, *tslot, 0);
 
-    if (warp == 0 && lane == 0) {
+    if (warp == 0 && elect_one()) {
         const uint16_t *x = half ? p.x1 : p.x0;
         bool ok = true;
         for (int c = 0; c < ntile + 6 && ok; ++c) {          // chunk c: positions 64 (tile0 - 3 + c) ..
@@ -563,7 +566,7 @@ __global__ void __launch_bounds__(WW_THREADS, 1) k_wgrad_win(const WgradWinParam
                 bulk_load(sDy + d * DYB + j * (WW_TILE * 16),
                           p.dy + ((size_t)j * p.rows + LEAD + (long)WW_TILE * (tile0 + i)) * 8, WW_TILE * 16, dF + 8 * d);
         }
-    } else if ((warp == 1 || warp == 2) && lane == 0) {
+    } else if ((warp == 1 || warp == 2) && elect_one()) {
         const uint32_t idesc = idesc_bf16(128, 64, 1, 1);
         const int g0 = (warp - 1) * 3;
         bool ok = true;
@@ -616,7 +619,7 @@ size_t conv_smem_bytes(const ConvParams &p)
 {
     const size_t upl = p.cg / 8 < 4 ? p.cg / 8 : 4;
     const size_t wbytes = p.resident ? (size_t)p.ngroups * p.taps * p.N * p.cg * 2 : (size_t)p.slots * p.N * upl * 16;
-    return 2 * upl * p.plane + wbytes + 64 + 16 * p.slots + 8 + 1024;
+    return p.stages * upl * p.plane + wbytes + 16 * p.stages + 32 + 16 * p.slots + 8 + 1024;
 }
 
 size_t wgrad_smem_bytes(const WgradParams &p)

@@ -36,6 +36,7 @@ struct ConvParams {
     int ngroups;           // 1, or 2 when the input is the concatenation of two tensors
     int N;                 // GEMM N = output channels (16 .. 128)
     int mt;                // 128-row M tiles per tile (one window)
+    int stages;            // window stages (one unit of up to 32 channels each)
     int slots;             // weight ring slots (streamed weights)
     int resident;          // 1: all weight blocks loaded once per CTA (no ring)
     uint32_t ncols;        // TMEM columns allocated

@@ -20,6 +20,19 @@ namespace nn {
 
 __device__ __forceinline__ uint32_t su32(const void *p) { return (uint32_t)__cvta_generic_to_shared(p); }
 
+// One thread of a converged warp, the same one every time.  A branch on it (and
+// on warp_index()) is one the compiler knows to be taken by whole warps up to
+// the election, so what a single thread computes there stays in uniform
+// registers, where tcgen05.mma wants its operands: 65 cycles per MMA (M = 128,
+// N = 64) from one issuing thread against 101 behind `lane == 0`.
+__device__ __forceinline__ bool elect_one()
+{
+    uint32_t r;
+    asm volatile("{\n .reg .pred e;\n elect.sync _|e, 0xffffffff;\n selp.u32 %0, 1, 0, e;\n}\n" : "=r"(r));
+    return r != 0;
+}
+__device__ __forceinline__ int warp_index() { return __shfl_sync(0xffffffffu, threadIdx.x >> 5, 0); }
+
 // ---------------------------------------------------------------- mbarrier
 __device__ __forceinline__ void mb_init(uint32_t bar, uint32_t count)
 {
