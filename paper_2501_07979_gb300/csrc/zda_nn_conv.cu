@@ -163,7 +163,7 @@ __device__ __forceinline__ void mb_arrive(uint32_t bar)
 }
 
 // Persistent, warp-specialised convolution.  Warp 0 (one lane) streams, per
-// tile and input unit, the bulk-copied window into one of two stages; the
+// tile and input unit, the bulk-copied window into one of two to four stages; the
 // weight blocks are either loaded once per CTA (resident: every layer whose
 // weights fit beside the two windows) or streamed per tap through a ring
 // (the concatenating layers); warp 1 (one lane) issues the MMAs
