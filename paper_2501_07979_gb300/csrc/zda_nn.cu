@@ -267,51 +267,67 @@ __global__ void __launch_bounds__(256) k_colsum(const uint16_t *g, long rows, lo
 
 // Layer gradient from the wgrad partials and the bias partials [nblk][cout]:
 // grads[w[co][t][ci]], grads[b[co]].  A block sums 64 neighbouring values of the
-// partials (a whole 256-byte line of every split) with 16 threads to a value;
-// the last block sums the biases.  Bound by the latency of its few rounds of
-// loads.  (Threads along c_in, each walking all splits alone: 20 us a layer,
-// 213 us of the 1.05 ms of a one-sample gradient.)
+// partials (a whole 256-byte line of every split), four to a thread and
+// LG_PARTS threads to a value, so a thread's ten or so 16-byte loads are all in
+// flight; the last block sums the biases.  Bound by that one round of loads
+// (30 MB of partials from L2).  One value per thread: 16 us a layer of a
+// 64-sample gradient, 9 now; threads along c_in that each walked all splits
+// alone: 20 us a layer of a one-sample gradient.
 // win = 0: [splits][ngroups][128][N] of k_wgrad_tc; 1: [tensors][splits][6][16][128][4] of k_wgrad_win.
-constexpr int LG_THREADS = 1024, LG_VALUES = 64, LG_PARTS = LG_THREADS / LG_VALUES;
+constexpr int LG_THREADS = 256, LG_VALUES = 64, LG_PARTS = LG_THREADS * 4 / LG_VALUES;
 __global__ void __launch_bounds__(LG_THREADS) k_layer_grad(const float *wpart, int win, int splits, int ngroups, int ntap_grp,
                                                            int cin_pad, int N, const float *bpart, int nblk, int cout,
                                                            int cin, int taps, float *grad)
 {
-    __shared__ float red[LG_THREADS];
-    const int lane = threadIdx.x % LG_VALUES, part = threadIdx.x / LG_VALUES;
+    __shared__ float red[LG_PARTS][LG_VALUES];
+    const int first4 = threadIdx.x * 4 % LG_VALUES, part = threadIdx.x * 4 / LG_VALUES;
     const bool bias = blockIdx.x + 1 == gridDim.x;
-    const long v = (long)blockIdx.x * LG_VALUES + lane;      // value of one split's partial (all tensors in turn)
     const int per = (win ? WW_GROUPS : ngroups) * 128 * N;   // values of a split
-    int co, t, ci;
-    size_t first = (size_t)v;
-    if (win) {
-        const int half = (int)(v / per), w = (int)(v % per), g = w / (128 * 64), row = w / 4 % 128;
-        co = w / 512 % 16 * 4 + w % 4;
-        t = g / 2 * 3 + ((g & 1) ? 2 : row / 64);
-        ci = half * 64 + row % 64;
-        if ((g & 1) && row >= 64) t = taps;                  // the unused second tap
-        first = (size_t)half * splits * per + w;
+    // where value v of a split (all tensors in turn) comes from and goes to; runs of four share tap and c_in
+    auto locate = [&](long v, size_t &from, int &co, int &t, int &ci) {
+        if (win) {
+            const int half = (int)(v / per), w = (int)(v % per), g = w / (128 * 64), row = w / 4 % 128;
+            co = w / 512 % 16 * 4 + w % 4;
+            t = (g & 1) && row >= 64 ? taps : g / 2 * 3 + ((g & 1) ? 2 : row / 64);   // taps: the unused second tap
+            ci = half * 64 + row % 64;
+            from = (size_t)half * splits * per + w;
+        } else {
+            const int row = (int)(v / N) % 128, g = (int)(v / (128 * N));
+            co = (int)(v % N);
+            t = g * ntap_grp + row / cin_pad;
+            ci = row % cin_pad;
+            from = (size_t)v;
+        }
+    };
+    float4 s = make_float4(0.f, 0.f, 0.f, 0.f);
+    if (bias) {
+        float *f = reinterpret_cast<float *>(&s);
+        for (int e = 0; e < 4; ++e)
+            if (first4 + e < cout)
+                for (int k = part; k < nblk; k += LG_PARTS) f[e] += __ldg(bpart + (size_t)k * cout + first4 + e);
     } else {
-        const int row = (int)(v / N) % 128, g = (int)(v / (128 * N));
-        co = (int)(v % N);
-        t = g * ntap_grp + row / cin_pad;
-        ci = row % cin_pad;
-    }
-    if (bias) co = lane;
-    const bool on = co < cout && (bias || (t < taps && ci < cin));
-    const float *src = bias ? bpart + lane : wpart + first;
-    const size_t stride = bias ? (size_t)cout : (size_t)per;
-    const int count = on ? (bias ? nblk : splits) : 0;
-    float s = 0.f;
+        size_t from;
+        int co, t, ci;
+        locate((long)blockIdx.x * LG_VALUES + first4, from, co, t, ci);
+        const float4 *src = reinterpret_cast<const float4 *>(wpart + from);
+        const int count = co < cout && t < taps && ci < cin ? splits : 0;
 #pragma unroll 10
-    for (int k = part; k < count; k += LG_PARTS) s += __ldg(src + k * stride);
-    red[threadIdx.x] = s;
-    __syncthreads();
-    if (part == 0 && on) {
-#pragma unroll
-        for (int q = 1; q < LG_PARTS; ++q) s += red[q * LG_VALUES + lane];
-        grad[bias ? (long)cout * taps * cin + co : ((long)co * taps + t) * cin + ci] = s;
+        for (int k = part; k < count; k += LG_PARTS) {
+            const float4 v = __ldg(src + (size_t)k * (per / 4));
+            s.x += v.x; s.y += v.y; s.z += v.z; s.w += v.w;
+        }
     }
+    *reinterpret_cast<float4 *>(&red[part][first4]) = s;
+    __syncthreads();
+    if (threadIdx.x >= LG_VALUES) return;
+    size_t from;
+    int co = threadIdx.x, t = 0, ci = 0;
+    if (!bias) locate((long)blockIdx.x * LG_VALUES + threadIdx.x, from, co, t, ci);
+    if (co >= cout || t >= taps || ci >= cin) return;
+    float sum = red[0][threadIdx.x];
+#pragma unroll
+    for (int q = 1; q < LG_PARTS; ++q) sum += red[q][threadIdx.x];
+    grad[bias ? (long)cout * taps * cin + co : ((long)co * taps + t) * cin + ci] = sum;
 }
 
 struct PackLayer {
@@ -432,7 +448,7 @@ struct zda_nn {
         size_t g[LEV][4];     // per level: gA, gB, gU, gS
     } o{};
     size_t wpart_floats = 0;
-    int bpart_blocks = 240;
+    int bpart_blocks = 240;      // at least WW_CTAS
     int adam_step = 0;
     long long launches = 0;
     int n_fwd = 0;
@@ -592,6 +608,7 @@ zda_status layer_grad(zda_nn *net, int li, int n, const uint16_t *x0, const uint
         p.x1 = x1;
         p.dy = g;
         p.partial = at<float>(net, net->o.wpart);
+        p.bias = at<float>(net, net->o.bpart);
         p.err = at<int>(net, net->o.err);
         p.wait_limit = 1 << 22;
         e = launch_wgrad_win(p, splits, s);
@@ -624,14 +641,18 @@ zda_status layer_grad(zda_nn *net, int li, int n, const uint16_t *x0, const uint
         e = launch_wgrad(p, splits, s);
     }
     if (e != cudaSuccess) return nn_fail(ZDA_ERR_CUDA, std::string("wgrad launch: ") + cudaGetErrorString(e));
-    // bias partials: blocks of at least 1024 positions per plane, so that small levels leave few of them
-    const int nblk = (int)std::max<long>(1, std::min<long>(net->bpart_blocks, P / 1024));
-    k_colsum<<<dim3(nblk, ldg / 8), 256, 0, s>>>(g, rows, P, l.cout, at<float>(net, net->o.bpart));
+    // bias partials: k_wgrad_win leaves one per block; else blocks of at least 1024 positions per plane, so that
+    // small levels leave few of them
+    int nblk = splits;
+    if (!win) {
+        nblk = (int)std::max<long>(1, std::min<long>(net->bpart_blocks, P / 1024));
+        k_colsum<<<dim3(nblk, ldg / 8), 256, 0, s>>>(g, rows, P, l.cout, at<float>(net, net->o.bpart));
+        net->launches++;
+    }
     k_layer_grad<<<(unsigned)((long)nrow * ldg / LG_VALUES) + 1, LG_THREADS, 0, s>>>(
         at<float>(net, net->o.wpart), win ? 1 : 0, splits, ngroups, ntap_grp, l.cin_pad, ldg,
-                                          at<float>(net, net->o.bpart), nblk, l.cout, l.cin, taps,
-                                          at<float>(net, net->o.grads) + l.off);
-    net->launches += 3;
+        at<float>(net, net->o.bpart), nblk, l.cout, l.cin, taps, at<float>(net, net->o.grads) + l.off);
+    net->launches += 2;
     e = cudaGetLastError();
     if (e != cudaSuccess) return nn_fail(ZDA_ERR_CUDA, std::string("gradient reduction: ") + cudaGetErrorString(e));
     return ZDA_OK;

@@ -508,7 +508,10 @@ __global__ void __launch_bounds__(WG_THREADS, 1)
 // behind its end too, for the steps that straddle it.
 // Roles (256 threads): warp 0 lane 0 producer, warps 1 and 2 lane 0 issue three
 // accumulators each, warp 3 owns TMEM; all warps store (0..3 the first three
-// accumulators, 4..7 the others).  Waits are bounded.
+// accumulators, 4..7 the others).  Until then warps 4..7 of the first tensor's
+// blocks add up the dY tiles in shared memory for the bias gradient, which
+// took a kernel of its own and a second read of dY (24 us at 64 x 128 x 128
+// positions).  Waits are bounded.
 __global__ void __launch_bounds__(WW_THREADS, 1) k_wgrad_win(const WgradWinParams p)
 {
     constexpr int RING = WW_SLOTS * WW_TILE, ROWS = RING + 16;
@@ -531,7 +534,7 @@ __global__ void __launch_bounds__(WW_THREADS, 1) k_wgrad_win(const WgradWinParam
         }
         for (int s = 0; s < WW_DY; ++s) {
             mb_init(dF + 8 * s, 1);
-            mb_init(dE + 8 * s, 2);
+            mb_init(dE + 8 * s, half ? 2 : 6);     // and one arrival per summing warp
         }
         mb_init(bDone, 2);
         *abort = 0;
@@ -593,6 +596,39 @@ __global__ void __launch_bounds__(WW_THREADS, 1) k_wgrad_win(const WgradWinParam
             tc_commit(dE + 8 * d);
         }
         if (ok) tc_commit(bDone);
+    } else if (warp >= 4 && half == 0) {
+        const int th = threadIdx.x - 128, plane = th >> 4, sub = th & 15;    // 16 threads to a plane of 8 channels
+        float acc[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+        bool ok = true;
+        for (int i = 0; i < ntile && ok; ++i) {
+            const int d = i % WW_DY;
+            ok = __all_sync(0xffffffffu, wait_or_abort(dF + 8 * d, (i / WW_DY) & 1, p.wait_limit, abort, p.err, 36));
+            if (!ok) break;
+            const uint4 *row = reinterpret_cast<const uint4 *>(smem + (sDy + d * DYB - raw)) + plane * WW_TILE + sub;
+            uint4 v[WW_TILE / 16];
+#pragma unroll
+            for (int k = 0; k < WW_TILE / 16; ++k) v[k] = row[16 * k];
+            __syncwarp();
+            if (lane == 0) mb_arrive(dE + 8 * d);
+#pragma unroll
+            for (int k = 0; k < WW_TILE / 16; ++k) {
+                const uint32_t w[4] = {v[k].x, v[k].y, v[k].z, v[k].w};
+#pragma unroll
+                for (int e = 0; e < 4; ++e) {
+                    acc[2 * e] += __uint_as_float(w[e] << 16);
+                    acc[2 * e + 1] += __uint_as_float(w[e] & 0xffff0000u);
+                }
+            }
+        }
+        __syncwarp();
+#pragma unroll
+        for (int e = 0; e < 8; ++e)
+            for (int o = 8; o > 0; o >>= 1) acc[e] += __shfl_xor_sync(0xffffffffu, acc[e], o);
+        if (sub == 0) {
+            float4 *out = reinterpret_cast<float4 *>(p.bias + split * 64 + plane * 8);
+            out[0] = make_float4(acc[0], acc[1], acc[2], acc[3]);
+            out[1] = make_float4(acc[4], acc[5], acc[6], acc[7]);
+        }
     }
     __syncwarp();
     const bool done = wait_or_abort(bDone, 0, p.wait_limit, abort, p.err, 35);

@@ -84,6 +84,7 @@ struct WgradWinParams {
     long rows;
     const uint16_t *x0, *x1, *dy;  // x1: second tensor of a concatenated input or null
     float *partial;        // [tensors][splits][6][64 / 4][128][4]
+    float *bias;           // [splits][64]: sums of dy over the blocks' positions
     int *err;
     int wait_limit;
 };
