@@ -870,7 +870,8 @@ static zda_status tile_h_maps(zda_zone &z)
 static bool uses_waits(const zda_zone &z) { return z.variant == 1 || (z.variant >= 3 && z.variant <= 5) || z.grid_run; }
 
 // Whether this run takes the resident step; the launches of the split step
-// run instead under a kernel chosen by zda_zone_set_kernel, under the event
+// run instead under a kernel chosen by zda_zone_set_kernel, on forward runs
+// whose final fields may have decayed (final_fields_decay), under the event
 // timing and the decay probe (both look between the launches of a step), and
 // where other work may run beside it (shared: a lens's branches, a stream
 // capture), because the resident step's blocks wait on one another.
@@ -1441,13 +1442,29 @@ zda_status zda_filter_project_backward(zda_zone *z, const float *rho, const floa
     return ZDA_OK;
 }
 
-zda_status zda_forward(zda_zone *z, const float *rho, double *focal_out, void *stream)
+// Whether the fields that a forward run ends with may have decayed to the run's rounding noise.  There two forms of
+// the step agree with the exact fields equally well but not with each other, so a run whose final fields the caller
+// may read keeps the split step's.  Over 1432 random zones the resident step's final fields were 2e-5 to 6e-4 away
+// from the split step's on 82 (the exact ones 3e-5 from both): all with cells of less than 0.03 wavelengths, or with
+// at most 1.5 wavelengths between the PMLs at cells of 0.05, none at 0.1; at the sizes let through at most 1e-5.
+// The monitor DFTs differ by at most 1.5e-6 on all of them.
+static bool final_fields_decay(const zda_zone &z)
+{
+    const zda_zone_desc &d = z.d;
+    double lam = 0;
+    for (double l : z.lambda) lam = std::max(lam, l);
+    const double cell = std::min(d.dr, d.dz) / lam;
+    const double open = std::min((d.n_r - d.pml_r_in - d.pml_r_out) * d.dr, (d.n_z - 2 * d.pml_z) * d.dz) / lam;
+    return cell < 0.08 && (cell < 0.04 || open < 1.55);
+}
+
+static zda_status forward_run(zda_zone *z, const float *rho, double *focal_out, void *stream, bool fields_read)
 {
     zda_status st = ready(z);
     if (st) return st;
     if (!rho || !focal_out) return fail(ZDA_ERR_ARG, "null pointer");
     cudaStream_t s = (cudaStream_t)stream;
-    st = forward_enqueue(*z, rho, s, false);
+    st = forward_enqueue(*z, rho, s, fields_read && final_fields_decay(*z));
     if (st) return st;
     st = check_wait_status(*z, s);
     if (st) return st;
@@ -1455,6 +1472,11 @@ zda_status zda_forward(zda_zone *z, const float *rho, double *focal_out, void *s
     if (st) return st;
     z->have_forward = true;
     return ZDA_OK;
+}
+
+zda_status zda_forward(zda_zone *z, const float *rho, double *focal_out, void *stream)
+{
+    return forward_run(z, rho, focal_out, stream, true);
 }
 
 zda_status zda_adjoint(zda_zone *z, const double *dI, float *grad_rho, void *stream)
@@ -1491,7 +1513,7 @@ zda_status zda_iteration(zda_zone *z, const float *rho, double *I_out, float *gr
         g_dev = P<float>(*z, z->L.g_rho);
     }
     std::vector<double> S(2 * z->nq), g(2 * z->nq);
-    st = zda_forward(z, rho_dev, S.data(), stream);
+    st = forward_run(z, rho_dev, S.data(), stream, false);     // the adjoint run overwrites its final fields
     if (st) return st;
     double I = 0;
     for (int q = 0; q < z->nq; ++q) {
