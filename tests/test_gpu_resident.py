@@ -154,3 +154,15 @@ def test_launches_of_the_split_step_stay_in_reach():
     z.set_energy_probe(20)
     S3 = z.forward(r)
     assert len(z.energy_trace()[0]) == spec.n_steps // 20 and _rel(S3, S) < 1e-5
+
+
+@pytest.mark.parametrize("cell,n_r,one_launch", [(0.1, 24, True), (0.05, 24, False), (0.05, 48, True), (0.03, 64, False)])
+def test_forward_runs_that_end_in_noise_keep_the_split_step(cell, n_r, one_launch):
+    """zda_forward leaves the one-launch run where the final fields may have decayed: fine cells, or few
+    wavelengths between the PMLs at medium ones."""
+    spec = zone_tiny(dr=cell, dz=cell, n_r=n_r, n_z=48, filter_radius=1.6 * cell, beta=3.0, wavelengths=(1.0,),
+                     pulse_sigma=0.4, pulse_t0=1.6, n_steps=300)
+    z = _zone(spec)
+    n0 = z.launches
+    z.forward(_dev(_rho(spec)))
+    assert (z.launches - n0 < 20) == one_launch
