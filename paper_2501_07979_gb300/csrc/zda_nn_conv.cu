@@ -608,8 +608,6 @@ __global__ void __launch_bounds__(WW_THREADS, 1) k_wgrad_win(const WgradWinParam
             uint4 v[WW_TILE / 16];
 #pragma unroll
             for (int k = 0; k < WW_TILE / 16; ++k) v[k] = row[16 * k];
-            __syncwarp();
-            if (lane == 0) mb_arrive(dE + 8 * d);
 #pragma unroll
             for (int k = 0; k < WW_TILE / 16; ++k) {
                 const uint32_t w[4] = {v[k].x, v[k].y, v[k].z, v[k].w};
@@ -619,6 +617,12 @@ __global__ void __launch_bounds__(WW_THREADS, 1) k_wgrad_win(const WgradWinParam
                     acc[2 * e + 1] += __uint_as_float(w[e] & 0xffff0000u);
                 }
             }
+            // The slot goes back to the bulk copies, which write through the async proxy: the values have to be in
+            // registers (the sums hold them there) and this thread's reads ordered before that proxy's writes.
+            asm volatile("" ::"f"(acc[0]), "f"(acc[1]), "f"(acc[2]), "f"(acc[3]), "f"(acc[4]), "f"(acc[5]), "f"(acc[6]), "f"(acc[7]));
+            fence_async_shared();
+            __syncwarp();
+            if (lane == 0) mb_arrive(dE + 8 * d);
         }
         __syncwarp();
 #pragma unroll

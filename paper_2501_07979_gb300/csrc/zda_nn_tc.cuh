@@ -61,6 +61,9 @@ __device__ __forceinline__ bool mb_wait(uint32_t bar, uint32_t parity, int limit
     return false;
 }
 
+// Orders this thread's reads and writes of shared memory before later ones of the async proxy (bulk copies, MMA).
+__device__ __forceinline__ void fence_async_shared() { asm volatile("fence.proxy.async.shared::cta;" ::: "memory"); }
+
 // ---------------------------------------------------------------- copies
 // Contiguous bulk copy (16-byte aligned addresses, size a multiple of 16).
 __device__ __forceinline__ void bulk_load(uint32_t dst, const void *src, uint32_t bytes, uint32_t bar)

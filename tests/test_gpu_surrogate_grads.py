@@ -52,3 +52,33 @@ def test_loss_is_the_mean_square(n):
     d = (y - t).double()
     assert abs(loss.item() - (d * d).mean().item()) < 1e-6 * (d * d).mean().item()
     assert _rel(dy.cpu().numpy(), (2 * d / d.numel()).cpu().numpy()) < 1e-6
+
+
+@pytest.mark.parametrize("seed", [0, 1])
+def test_gradients_of_many_positions_are_sound_and_repeat(seed):
+    """64 copies of one 128 x 128 sample: every block of k_wgrad_win streams a hundred tiles through its rings, so a
+    dY tile whose slot is refilled before the bias sums have read it shows, as bits that differ from pass to pass
+    and as bias entries off by 1e-3.  Exact-structure network as above, so a layer's bias gradient is 64 times the
+    sample's FP64 sum of the layer's output gradient: 480 FP32 additions deep over values that cancel, about 1e-7
+    relative, held to 1e-6; the weights to 5e-5 (an accumulator in tensor memory takes 448 steps of 2^-24 at most,
+    2.7e-5, then 23 more additions)."""
+    ic, oc, H, W, B = 1, 24, 128, 128, 64
+    ps = _perm_params(ic, oc, (True, False, True))
+    r = np.random.default_rng(seed)
+    x = S.bf16(r.uniform(0.05, 1, (1, H, W, ic)))
+    dy = S.bf16(r.standard_normal((1, H, W, oc)))
+    net = _net(H, W, ic, oc, B)
+    net.set_params(S.flatten(ps).astype(np.float32))
+    net.forward(torch.tensor(x, dtype=torch.float32, device="cuda:0").expand(B, -1, -1, -1))
+    d = torch.tensor(dy, dtype=torch.float32, device="cuda:0").expand(B, -1, -1, -1).contiguous()
+    net.backward(d)
+    first = net.grads()
+    for k in range(100):
+        net.backward(d)
+        assert torch.equal(net.grads().view(torch.int32), first.view(torch.int32)), k
+    net.check()
+    want, _ = S.backward(ps, S.forward(ps, x, rounding=True)[1], dy)
+    got = S.unflatten(first.cpu().numpy().astype(np.float64), ic, oc)
+    for (name, *_), (gw, gb), (ww, wb) in zip(S.layer_table(ic, oc), got, want):
+        assert _rel(gb, B * wb) < 1e-6, name
+        assert _rel(gw, B * ww) < 5e-5, name
