@@ -879,6 +879,7 @@ static bool resident_route(zda_zone &z, const zda::StepParams &p, bool shared)
 {
     if (shared || !z.kernel_default || z.variant != 0 || z.time_every > 0 || !z.mail_bytes) return false;
     if (z.probe_every > 0 && p.src_mode == zda::SRC_PLANE_WAVE) return false;
+    if (z.d.n_steps < 2) return false;       // (see resident_loop)
     make_resident_plan(z);
     return z.res.blocks() > 0;
 }
@@ -1034,11 +1035,15 @@ static zda_status resident_loop(zda_zone &z, zda::StepParams &p, cudaStream_t s,
     std::lock_guard<std::mutex> guard(turn.m);
     if (turn.last) CUDA_TRY(cudaStreamWaitEvent(s, turn.last, 0));
     else CUDA_TRY(cudaEventCreateWithFlags(&turn.last, cudaEventDisableTiming));
-    // one launch per 4096 steps (a multiple of DFT_BLOCK): a run of any length stays preemptible
-    const int chunk = 4096;
-    for (int n = 0; n < z.d.n_steps; n += chunk) {
-        const cudaError_t e = zda::launch_resident(z.res, p, n, std::min(n + chunk, z.d.n_steps), z.d.n_steps, mail,
-                                                   P<int>(z, z.L.status) + 1, z.wait_limit, z.inject_timeout, s);
+    // One launch per 4096 steps (a multiple of DFT_BLOCK): a run of any length stays preemptible.  No launch of one
+    // step: a brick reads its neighbours' state as it begins and writes its own as it ends, and what tells it that
+    // they have read it are their packets of the step before the last.
+    const int chunk = 4096, T = z.d.n_steps;
+    for (int n = 0, m; n < T; n = m) {
+        m = std::min(n + chunk, T);
+        if (T - m == 1) m -= zda::DFT_BLOCK;
+        const cudaError_t e = zda::launch_resident(z.res, p, n, m, T, mail, P<int>(z, z.L.status) + 1, z.wait_limit,
+                                                   z.inject_timeout, s);
         if (n == 0 && e == cudaErrorCooperativeLaunchTooLarge) {
             (void)cudaGetLastError();
             return ZDA_OK;

@@ -166,3 +166,22 @@ def test_forward_runs_that_end_in_noise_keep_the_split_step(cell, n_r, one_launc
     n0 = z.launches
     z.forward(_dev(_rho(spec)))
     assert (z.launches - n0 < 20) == one_launch
+
+
+@pytest.mark.parametrize("n_steps", [1, 2, 4096, 4097, 4098])
+def test_no_launch_of_a_single_step(n_steps):
+    """A brick overwrites its state as its launch ends and its neighbours read it as theirs begin: only with two steps
+    between is the second behind the first.  Runs of one step, and of one more than a launch takes, against the split
+    step (FP32 rounding: 1e-5; the fields of the long runs have decayed, so their DFTs are held)."""
+    spec = zone_tiny(**{**BASE, "n_steps": n_steps, "pulse_t0": 0.0})
+    rho = _dev(_rho(spec))
+    a, b = _zone(spec), _zone(spec)
+    b.set_kernel(0, 4, 0)
+    n0 = a.launches
+    Sa = a.forward(rho)
+    assert a.launches - n0 < 20
+    Sb = b.forward(rho)
+    assert _rel(Sa, Sb) < 1e-5
+    assert _rel(a.monitor_dft().cpu(), b.monitor_dft().cpu()) < 1e-5
+    if n_steps < 3:
+        assert _rel(a.fields().cpu(), b.fields().cpu()) < 1e-5
