@@ -182,6 +182,7 @@ def test_no_launch_of_a_single_step(n_steps):
     assert a.launches - n0 < 20
     Sb = b.forward(rho)
     assert _rel(Sa, Sb) < 1e-5
-    assert _rel(a.monitor_dft().cpu(), b.monitor_dft().cpu()) < 1e-5
-    if n_steps < 3:
+    if n_steps < 3:                                      # nothing has reached the monitor yet
         assert _rel(a.fields().cpu(), b.fields().cpu()) < 1e-5
+    else:
+        assert _rel(a.monitor_dft().cpu(), b.monitor_dft().cpu()) < 1e-5
