@@ -103,7 +103,7 @@ struct zda_zone {
     int wait_limit = 1 << 22, inject_timeout = 0;   // bounded waits of the fused, tiled and resident steps
     bool pair_kernels = true;       // split step: two z-cells per thread where the grid allows
     int rpml = 0;                   // r-PML form (zda_zone_set_radial_pml)
-    int last_parity = 0;            // fused runs: which buffer holds the final fields
+    int last_parity = 0;            // which field buffer the last run left its final fields in (0 but for fused runs)
     int probe_every = 0, probe_n = 0;   // decay probe of forward runs: sampling period, samples of the last run
     // optional CUDA-event timing of every `time_every`-th H/E launch pair
     int time_every = 0;
@@ -1576,7 +1576,7 @@ zda_status zda_copy_fields(zda_zone *z, float *out, void *stream)
     if (st) return st;
     if (!out) return fail(ZDA_ERR_ARG, "null pointer");
     const size_t n = 6 * (size_t)z->d.n_r * z->d.n_phi * z->d.n_z * sizeof(float2);
-    const size_t off = ((z->variant == 1 || z->variant == 3 || z->variant == 6) && z->last_parity) ? z->L.fields2 : z->L.fields;
+    const size_t off = z->last_parity ? z->L.fields2 : z->L.fields;
     CUDA_TRY(cudaMemcpyAsync(out, z->ws + off, n, cudaMemcpyDeviceToDevice, (cudaStream_t)stream));
     return ZDA_OK;
 }
@@ -1830,6 +1830,7 @@ struct zda_lens {
     bool use_graph = true;
     cudaGraphExec_t g_fwd = nullptr, g_adj = nullptr;
     std::vector<std::vector<long long>> stamp_fwd, stamp_adj;
+    std::vector<int> end_fwd, end_adj;     // last_parity of the zones after each graph: a replay runs no host code
     std::vector<cudaStream_t> streams;     // [0] capture / join stream, [1 + z] zone branches
     std::vector<cudaEvent_t> events;       // [0] fork, [1 + z] joins
     bool have_forward = false;
@@ -1884,7 +1885,7 @@ static zda_status lens_branches(zda_lens &L, F &&per_zone)
 
 template <class F>
 static zda_status lens_run(zda_lens &L, cudaGraphExec_t &exec, std::vector<std::vector<long long>> &stamp,
-                           cudaStream_t user, F &&body)
+                           std::vector<int> &ends, cudaStream_t user, F &&body)
 {
     cudaStream_t s0 = L.streams[0];
     if (!L.use_graph) {
@@ -1915,9 +1916,14 @@ static zda_status lens_run(zda_lens &L, cudaGraphExec_t &exec, std::vector<std::
         cudaGraphDestroy(g);
         if (e != cudaSuccess) { exec = nullptr; return fail(ZDA_ERR_CUDA, std::string("graph instantiate: ") + cudaGetErrorString(e)); }
         stamp.clear();
-        for (zda_zone *z : L.zones) stamp.push_back(zone_stamp(*z));
+        ends.clear();
+        for (zda_zone *z : L.zones) {
+            stamp.push_back(zone_stamp(*z));
+            ends.push_back(z->last_parity);
+        }
     }
     CUDA_TRY(cudaGraphLaunch(exec, user));
+    for (size_t z = 0; z < L.zones.size(); ++z) L.zones[z]->last_parity = ends[z];
     L.launches++;
     return ZDA_OK;
 }
@@ -2014,7 +2020,7 @@ zda_status zda_lens_forward(zda_lens *L, const float *const *rho, double *focal_
         CUDA_TRY(cudaGetLastError());
         return ZDA_OK;
     };
-    zda_status st = lens_run(*L, L->g_fwd, L->stamp_fwd, s, body);
+    zda_status st = lens_run(*L, L->g_fwd, L->stamp_fwd, L->end_fwd, s, body);
     if (st) return st;
     int flag = 0;
     CUDA_TRY(cudaMemcpyAsync(focal_out, L->ws + lens_ws_S(*L), L->nq * sizeof(double2), cudaMemcpyDeviceToHost, s));
@@ -2057,7 +2063,7 @@ zda_status zda_lens_adjoint(zda_lens *L, const double *dI, float *const *grad_rh
             return adjoint_enqueue(Z, P<float>(Z, Z.L.g_rho), sz, true);
         });
     };
-    zda_status st = lens_run(*L, L->g_adj, L->stamp_adj, s, body);
+    zda_status st = lens_run(*L, L->g_adj, L->stamp_adj, L->end_adj, s, body);
     if (st) return st;
     for (size_t z = 0; z < L->zones.size(); ++z) {
         zda_zone *Z = L->zones[z];

@@ -109,3 +109,31 @@ def test_two_step_refuses_what_it_does_not_implement():
             z.set_radial_pml(1)
         with pytest.raises(ZdaError, match="ZDA_ERR_ARG"):
             z.set_kernel(6, 16, 0)
+
+
+@pytest.mark.parametrize("use_graph", [True, False])
+@pytest.mark.parametrize("kernel", [(6, 16, 0), (3, 8, 0), (1, 2, 0)])
+def test_final_fields_of_a_replayed_lens_run(kernel, use_graph):
+    """An odd number of launches leaves the fields in the second buffer, also where the run was a replayed graph and
+    another run of the zone came in between; and a kernel chosen after a run does not move them."""
+    from paper_2501_07979_gb300.lens import Lens
+    spec = _spec("tiny").replace(n_steps=302 if kernel[0] == 6 else 301)
+    rho = _dev(smoothed_rho(spec.n_r_design, spec.n_phi, 8, mode="minmax"))
+    z = _zone(spec, *kernel)
+    lens = Lens([z], use_graph=use_graph)
+    lens.forward([rho])
+    want = z.fields().clone()
+    z.time_steps(40)
+    lens.forward([rho])
+    assert torch.equal(torch.view_as_real(z.fields()), torch.view_as_real(want))
+    z.set_kernel(0, 4, 0)
+    assert torch.equal(torch.view_as_real(z.fields()), torch.view_as_real(want))
+
+
+def test_final_fields_outlive_a_change_of_the_radial_pml():
+    spec = zone_patch(200.0, 38)
+    z = _zone(spec)
+    z.forward(_dev(smoothed_rho(spec.n_r_design, spec.n_phi, 9, mode="minmax")))
+    want = z.fields().clone()
+    z.set_radial_pml(1)
+    assert torch.equal(torch.view_as_real(z.fields()), torch.view_as_real(want))
