@@ -99,7 +99,7 @@ struct zda_zone {
     zda::ResidentPlan res;
     int res_form = -1;
     size_t mail_bytes = 0;
-    bool grid_run = false;          // the last run's bricks waited on one another through memory
+    bool waited = false;            // the last run launched kernels whose device-side waits are bounded
     int wait_limit = 1 << 22, inject_timeout = 0;   // bounded waits of the fused, tiled and resident steps
     bool pair_kernels = true;       // split step: two z-cells per thread where the grid allows
     int rpml = 0;                   // r-PML form (zda_zone_set_radial_pml)
@@ -866,9 +866,6 @@ static zda_status tile_h_maps(zda_zone &z)
     return ZDA_OK;
 }
 
-// kernels with bounded device-side waits report a timeout through the error word
-static bool uses_waits(const zda_zone &z) { return z.variant == 1 || (z.variant >= 3 && z.variant <= 5) || z.grid_run; }
-
 // Whether this run takes the resident step; the launches of the split step
 // run instead under a kernel chosen by zda_zone_set_kernel, on forward runs
 // whose final fields may have decayed (final_fields_decay), under the event
@@ -1052,7 +1049,7 @@ static zda_status resident_loop(zda_zone &z, zda::StepParams &p, cudaStream_t s,
         z.launches++;
     }
     CUDA_TRY(cudaEventRecord(turn.last, s));
-    z.grid_run = true;
+    z.waited = true;
     z.last_parity = 0;
     *done = true;
     return ZDA_OK;
@@ -1061,7 +1058,7 @@ static zda_status resident_loop(zda_zone &z, zda::StepParams &p, cudaStream_t s,
 static zda_status time_loop(zda_zone &z, zda::StepParams &p, cudaStream_t s, bool shared)
 {
     const int R = (int)z.ev_pending.size();
-    z.grid_run = false;
+    z.waited = false;
     if (resident_route(z, p, shared)) {
         bool done = false;
         const zda_status st = resident_loop(z, p, s, &done);
@@ -1070,6 +1067,7 @@ static zda_status time_loop(zda_zone &z, zda::StepParams &p, cudaStream_t s, boo
     // (the decay probe compares the states around a step: it takes the split step)
     if (z.variant == 6 && !(z.probe_every > 0 && p.src_mode == zda::SRC_PLANE_WAVE)) return two_step_loop(z, p, s);
     if (z.variant == 3) {
+        z.waited = true;
         zda_status st = tile_maps(z);
         if (st) return st;
         const bool dft = p.des || p.mon;
@@ -1111,6 +1109,7 @@ static zda_status time_loop(zda_zone &z, zda::StepParams &p, cudaStream_t s, boo
         return ZDA_OK;
     }
     if (z.variant == 1) {
+        z.waited = true;
         zda::FusedParams f[2] = {fused_params(z, p, 0), fused_params(z, p, 1)};
         // timed samples: [stream kernel] between events 0 and 1, [DFT kernel] between 1 and 2
         for (int n = 0; n < z.d.n_steps; ++n) {
@@ -1154,6 +1153,7 @@ static zda_status time_loop(zda_zone &z, zda::StepParams &p, cudaStream_t s, boo
     zda::TileParams etp{};
     int enrc = 1;
     if (etile) {
+        z.waited = true;
         zda_status st = tile_e_maps(z);
         if (st) return st;
         const size_t ncell = (size_t)z.d.n_r * z.d.n_phi * z.d.n_z;
@@ -1498,7 +1498,7 @@ zda_status zda_adjoint(zda_zone *z, const double *dI, float *grad_rho, void *str
     CUDA_TRY(cudaStreamIsCapturing(s, &cap));
     st = adjoint_enqueue(*z, grad_rho, s, cap != cudaStreamCaptureStatusNone);
     if (st) return st;
-    if (uses_waits(*z)) return check_wait_status(*z, s);
+    if (z->waited) return check_wait_status(*z, s);
     return ZDA_OK;
 }
 
@@ -1830,7 +1830,9 @@ struct zda_lens {
     bool use_graph = true;
     cudaGraphExec_t g_fwd = nullptr, g_adj = nullptr;
     std::vector<std::vector<long long>> stamp_fwd, stamp_adj;
-    std::vector<int> end_fwd, end_adj;     // last_parity of the zones after each graph: a replay runs no host code
+    // what each graph leaves of the zones' last run (a replay runs no host code)
+    struct RunEnd { int parity; bool waited; };
+    std::vector<RunEnd> end_fwd, end_adj;
     std::vector<cudaStream_t> streams;     // [0] capture / join stream, [1 + z] zone branches
     std::vector<cudaEvent_t> events;       // [0] fork, [1 + z] joins
     bool have_forward = false;
@@ -1885,7 +1887,7 @@ static zda_status lens_branches(zda_lens &L, F &&per_zone)
 
 template <class F>
 static zda_status lens_run(zda_lens &L, cudaGraphExec_t &exec, std::vector<std::vector<long long>> &stamp,
-                           std::vector<int> &ends, cudaStream_t user, F &&body)
+                           std::vector<zda_lens::RunEnd> &ends, cudaStream_t user, F &&body)
 {
     cudaStream_t s0 = L.streams[0];
     if (!L.use_graph) {
@@ -1919,11 +1921,14 @@ static zda_status lens_run(zda_lens &L, cudaGraphExec_t &exec, std::vector<std::
         ends.clear();
         for (zda_zone *z : L.zones) {
             stamp.push_back(zone_stamp(*z));
-            ends.push_back(z->last_parity);
+            ends.push_back({z->last_parity, z->waited});
         }
     }
     CUDA_TRY(cudaGraphLaunch(exec, user));
-    for (size_t z = 0; z < L.zones.size(); ++z) L.zones[z]->last_parity = ends[z];
+    for (size_t z = 0; z < L.zones.size(); ++z) {
+        L.zones[z]->last_parity = ends[z].parity;
+        L.zones[z]->waited = ends[z].waited;
+    }
     L.launches++;
     return ZDA_OK;
 }
@@ -2027,7 +2032,7 @@ zda_status zda_lens_forward(zda_lens *L, const float *const *rho, double *focal_
     CUDA_TRY(cudaMemcpyAsync(&flag, status, sizeof(int), cudaMemcpyDeviceToHost, s));
     CUDA_TRY(cudaStreamSynchronize(s));
     for (zda_zone *Z : L->zones) {
-        if (uses_waits(*Z)) {
+        if (Z->waited) {
             st = check_wait_status(*Z, s);
             if (st) return st;
         }
@@ -2073,7 +2078,7 @@ zda_status zda_lens_adjoint(zda_lens *L, const double *dI, float *const *grad_rh
     }
     CUDA_TRY(cudaStreamSynchronize(s));
     for (zda_zone *Z : L->zones)
-        if (uses_waits(*Z)) {
+        if (Z->waited) {
             st = check_wait_status(*Z, s);
             if (st) return st;
         }

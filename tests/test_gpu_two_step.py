@@ -11,7 +11,7 @@ import pytest
 import torch
 
 import oracle as O
-from zda_inputs import smoothed_rho, zone_patch, zone_tiny
+from zda_inputs import rho_for, smoothed_rho, zone_cfg2, zone_patch, zone_tiny
 
 pytestmark = pytest.mark.gpu
 
@@ -137,3 +137,26 @@ def test_final_fields_outlive_a_change_of_the_radial_pml():
     want = z.fields().clone()
     z.set_radial_pml(1)
     assert torch.equal(torch.view_as_real(z.fields()), torch.view_as_real(want))
+
+
+@pytest.mark.parametrize("use_graph", [True, False])
+def test_a_timeout_under_the_decay_probe_is_reported_by_the_lens(use_graph):
+    """Under the decay probe a large default zone runs its E updates on TMA tiles, whose waits are bounded: the lens
+    reads their error word, in the captured run and in a replayed one, and not that of a run without the probe."""
+    from paper_2501_07979_gb300 import ZdaError
+    from paper_2501_07979_gb300.lens import Lens
+    spec = zone_cfg2(n_steps=300)
+    rho = _dev(rho_for(spec, 2))
+    z = _zone(spec)
+    assert z.get_kernel()[0] == 6
+    lens = Lens([z], use_graph=use_graph)
+    z.set_energy_probe(50)
+    z.set_wait_limit(1000, inject_timeout=True)
+    for _ in range(2):
+        with pytest.raises(ZdaError, match="ZDA_ERR_TIMEOUT"):
+            lens.forward([rho])
+    z.set_energy_probe(0)
+    S = lens.forward([rho])                              # two-step launches: nothing waits
+    z.set_energy_probe(50)
+    z.set_wait_limit(1 << 22)
+    assert _rel(lens.forward([rho]), S) < 1e-5
