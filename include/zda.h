@@ -159,7 +159,9 @@ zda_status zda_forward(zda_zone *zone, const float *rho_dev, double *focal_out_h
  * complex doubles (dI/dRe S_q, dI/dIm S_q) for any real objective I(S);
  * grad_rho_dev [n_r_design][n_phi] floats receives dI/drho.  Requires a
  * preceding zda_forward with the same rho (ZDA_ERR_STATE otherwise).  With
- * the fused step it synchronises the stream to report wait timeouts. */
+ * a step whose device-side waits are bounded (variants 1, 3, 4, 5 and the
+ * one-launch run of small zones) it synchronises the stream to learn of
+ * timeouts. */
 zda_status zda_adjoint(zda_zone *zone, const double *dI_dfocal_host, float *grad_rho_dev, void *stream);
 
 /* One TopOpt iteration of the summed focal intensity I = 2 sum |S_q|^2:
@@ -285,12 +287,15 @@ zda_status zda_zone_time_steps(zda_zone *zone, int steps, double *ms_out_host, v
 /* The fused and tiled steps (variants 1, 3, 4, 5) wait on shared-memory
  * barriers for their staged copies, the one-launch run of a small zone on
  * its neighbour blocks' halos; every wait gives up after `polls` polls
- * (default 4194304; variants 3 to 5 also after one second), sets an error
- * word and lets the kernel finish, and the call then returns
- * ZDA_ERR_TIMEOUT (zda_forward, zda_adjoint and zda_iteration synchronise
- * their stream to read it).  inject_timeout != 0 is for tests of that path:
- * variant 1 also waits, per radius, on a barrier that nothing completes;
- * variants 3, 4 and 5 once per thread block before their first radius. */
+ * (default 4194304; variants 3 to 5 also after one second, the one-launch
+ * run after two), sets an error word and lets the kernel finish.  A
+ * one-launch run that gave up is repeated by the split step within the call;
+ * after any other such run, and where the timeout was injected, the call
+ * returns ZDA_ERR_TIMEOUT.  zda_forward, zda_adjoint and zda_iteration
+ * synchronise their stream to read the word.  inject_timeout != 0 is for
+ * tests of that path: variant 1 also waits, per radius, on a barrier that
+ * nothing completes; variants 3, 4 and 5 once per thread block before their
+ * first radius; the one-launch run on halos that nothing sends. */
 zda_status zda_zone_set_wait_limit(zda_zone *zone, int polls, int inject_timeout);
 
 /* Kernel timing with CUDA events recorded on the launching stream: with

@@ -1228,6 +1228,13 @@ static zda_status check_wait_status(zda_zone &z, cudaStream_t s)
     return ZDA_OK;
 }
 
+// A one-launch run (of the variants without waits the only one that has them) that gave up waiting, because something
+// kept its blocks off the SMs or the caller's bound is short, is repeated by the launches of the split step.
+static bool repeat_by_split_step(const zda_zone &z, zda_status st)
+{
+    return st == ZDA_ERR_TIMEOUT && z.variant == 0 && !z.inject_timeout;
+}
+
 // focal kernels: S (workspace) and the non-finite flag (status[0])
 static zda_status focal_enqueue(zda_zone &z, const float2 *mon, cudaStream_t s)
 {
@@ -1472,6 +1479,10 @@ static zda_status forward_run(zda_zone *z, const float *rho, double *focal_out, 
     st = forward_enqueue(*z, rho, s, fields_read && final_fields_decay(*z));
     if (st) return st;
     st = check_wait_status(*z, s);
+    if (repeat_by_split_step(*z, st)) {
+        st = forward_enqueue(*z, rho, s, true);
+        if (st == ZDA_OK) st = check_wait_status(*z, s);
+    }
     if (st) return st;
     st = focal_finish(*z, focal_out, s);
     if (st) return st;
@@ -1498,8 +1509,9 @@ zda_status zda_adjoint(zda_zone *z, const double *dI, float *grad_rho, void *str
     CUDA_TRY(cudaStreamIsCapturing(s, &cap));
     st = adjoint_enqueue(*z, grad_rho, s, cap != cudaStreamCaptureStatusNone);
     if (st) return st;
-    if (z->waited) return check_wait_status(*z, s);
-    return ZDA_OK;
+    if (!z->waited) return ZDA_OK;
+    st = check_wait_status(*z, s);
+    return repeat_by_split_step(*z, st) ? adjoint_enqueue(*z, grad_rho, s, true) : st;
 }
 
 zda_status zda_iteration(zda_zone *z, const float *rho, double *I_out, float *grad_rho, int host_buffers,
@@ -1699,12 +1711,9 @@ zda_status zda_zone_get_radial_pml(const zda_zone *z, int *form)
     return ZDA_OK;
 }
 
-zda_status zda_zone_time_steps(zda_zone *z, int steps, double *ms_out, void *stream)
+static zda_status time_steps_run(zda_zone *z, int steps, double *ms_out, cudaStream_t s, bool shared)
 {
-    zda_status st = ready(z);
-    if (st) return st;
-    if (steps < 1 || !ms_out) return fail(ZDA_ERR_ARG, "bad argument");
-    cudaStream_t s = (cudaStream_t)stream;
+    zda_status st = ZDA_OK;
     z->have_forward = false;                 // the fields are overwritten
     zda::StepParams p = step_params(*z);
     p.src_mode = zda::SRC_NONE;
@@ -1719,7 +1728,7 @@ zda_status zda_zone_time_steps(zda_zone *z, int steps, double *ms_out, void *str
     z->d.n_steps = steps;
     z->time_every = 0;
     cudaError_t e = cudaEventRecord(a, s);
-    if (e == cudaSuccess) st = time_loop(*z, p, s, false);
+    if (e == cudaSuccess) st = time_loop(*z, p, s, shared);
     if (e == cudaSuccess && st == ZDA_OK) e = cudaEventRecord(b, s);
     if (e == cudaSuccess && st == ZDA_OK) e = cudaEventSynchronize(b);
     float ms = 0.f;
@@ -1732,6 +1741,17 @@ zda_status zda_zone_time_steps(zda_zone *z, int steps, double *ms_out, void *str
     if (e != cudaSuccess) return fail(ZDA_ERR_CUDA, std::string("timing: ") + cudaGetErrorString(e));
     *ms_out = ms;
     return check_wait_status(*z, s);
+}
+
+zda_status zda_zone_time_steps(zda_zone *z, int steps, double *ms_out, void *stream)
+{
+    zda_status st = ready(z);
+    if (st) return st;
+    if (steps < 1 || !ms_out) return fail(ZDA_ERR_ARG, "bad argument");
+    st = time_steps_run(z, steps, ms_out, (cudaStream_t)stream, false);
+    if (!repeat_by_split_step(*z, st)) return st;
+    CUDA_TRY(cudaMemsetAsync(P<int>(*z, z->L.status) + 1, 0, sizeof(int), (cudaStream_t)stream));
+    return time_steps_run(z, steps, ms_out, (cudaStream_t)stream, true);
 }
 
 zda_status zda_zone_set_wait_limit(zda_zone *z, int polls, int inject_timeout)

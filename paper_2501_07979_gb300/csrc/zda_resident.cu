@@ -30,7 +30,7 @@
 // Packets are double-buffered by step parity; neighbours read from each other,
 // so a packet is only overwritten after its reader has sent the step in
 // between.  Waits are bounded; a brick that gives up sets the error word and
-// leaves.  (As one thread-block cluster, with the halo read from the
+// leaves, and the caller repeats the run by the split step.  (As one thread-block cluster, with the halo read from the
 // neighbours' shared memory, a step of the 24 x 8 x 40 zone took 4.1 us: the
 // cluster barriers cost as much as the packets and 16 SMs hold too few warps.)
 //
@@ -758,15 +758,14 @@ __global__ void __launch_bounds__(C == 1 ? RES_THREADS_1 : RES_THREADS, 1) k_res
                             E[r[u].y & 0x3fffffffu] = r[u].y >> 30 ? turn(p.bloch, v) : v;
                             open &= ~(1 << u);
                         }
-                    if (open && (++polls & 63) == 0) {       // bounded: two seconds, or another brick gave up
+                    if (!open) break;
+                    bad = ++polls >= q.wait_limit;           // bounded: the polls, two seconds, or another brick gave up
+                    if ((polls & 63) == 0) {
                         const u64 t = now_ns();
                         if (!since) since = t;
-                        if ((q.inject_timeout && polls >= q.wait_limit) || t - since > 2000000000ull ||
-                            *(volatile int *)q.err) {
-                            bad = true;
-                            break;
-                        }
+                        bad = bad || t - since > 2000000000ull || *(volatile int *)q.err;
                     }
+                    if (bad) break;
                 }
             }
         }

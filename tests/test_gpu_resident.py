@@ -186,3 +186,27 @@ def test_no_launch_of_a_single_step(n_steps):
         assert _rel(a.fields().cpu(), b.fields().cpu()) < 1e-5
     else:
         assert _rel(a.monitor_dft().cpu(), b.monitor_dft().cpu()) < 1e-5
+
+
+@pytest.mark.parametrize("name", ["tiny", "two_cells"])
+def test_a_run_that_gives_up_waiting_is_repeated_by_the_split_step(name):
+    """One poll is less than a neighbour's packet takes: the run gives up, and the call's result is the split step's,
+    bit for bit, for every entry point that may take the one-launch run."""
+    spec = _spec(name)
+    rho = _dev(_rho(spec))
+    a, b = _zone(spec), _zone(spec)
+    b.set_kernel(0, 2, 0)
+    want = a.forward(rho)
+    a.set_wait_limit(1)
+    n0 = a.launches
+    S, Sb = a.forward(rho), b.forward(rho)
+    assert a.launches - n0 > 2 * spec.n_steps and np.array_equal(S, Sb)
+    assert torch.equal(a.monitor_dft(), b.monitor_dft()) and torch.equal(a.fields(), b.fields())
+    assert torch.equal(a.adjoint(4.0 * S), b.adjoint(4.0 * S))
+    (Ia, ga), (Ib, gb) = a.iteration(rho), b.iteration(rho)
+    assert Ia == Ib and torch.equal(ga, gb)
+    n0 = a.launches
+    assert a.time_steps(50) > 0 and a.launches - n0 >= 100
+    a.set_wait_limit(1 << 22)
+    n0 = a.launches
+    assert np.array_equal(a.forward(rho), want) and a.launches - n0 < 20
