@@ -184,7 +184,7 @@ __global__ void __launch_bounds__(NT, NT > 192 ? 1 : 2) k_two(const __grid_const
     for (int t = tid; t < ie - ib + 4; t += blockDim.x) {
         const int i = min(max(ib - 2 + t, 0), nr - 1);
         const float irn = p.t.inv_r_n[i], irh = p.t.inv_r_h[i];
-        const float hA = -dt * irn * p.inv_dphi, hB = -irh * p.inv_dphi, eA = irh * p.inv_dphi, eB = -irn * p.inv_dphi;
+        const float hA = irn * p.inv_dphi, hB = -irh * p.inv_dphi, eA = irh * p.inv_dphi, eB = -irn * p.inv_dphi;
         tab[4 * t] = make_float4(hA, hA, hB, hB);
         tab[4 * t + 1] = make_float4(0.5f * irh, 0.5f * irh, 0.f, 0.f);
         tab[4 * t + 2] = make_float4(eA, eA, eB, eB);
@@ -205,7 +205,8 @@ __global__ void __launch_bounds__(NT, NT > 192 ? 1 : 2) k_two(const __grid_const
     const size_t plane = (size_t)nr * nphi, ndes = p.des ? plane * p.des_nk : 0;
     const bool hist = own && ((p.des && k + 1 >= p.des_k0 && k < p.des_k0 + p.des_nk) || (p.mon && (p.mon_k == k || p.mon_k == k + 1)));
 
-    const float2 c_dz = both(p.inv_dz), c_dr = both(p.inv_dr), c_dt = both(dt), c_dtdz = both(dt * p.inv_dz);
+    const float2 c_dz = both(p.inv_dz), c_ndz = both(-p.inv_dz), c_dr = both(p.inv_dr);
+    const float2 c_dt = both(dt), c_ndt = both(-dt);
     auto rslab = [&](int i) { return i < p.pr_in ? i >= 0 : (i >= nr - p.pr_out && i < nr); };
     auto rx_at = [&](int i) {                      // the pair in the r-slab arrays
         const int ir = i < p.pr_in ? i : i - (nr - p.pr_in - p.pr_out);
@@ -249,14 +250,13 @@ __global__ void __launch_bounds__(NT, NT > 192 ? 1 : 2) k_two(const __grid_const
         for (int u = 0; u < 2; ++u) {
             const float2 dzp = psub(u ? ep_k : e.p.a[1], e.p.a[u]), dzr = psub(u ? er_k : e.r.a[1], e.r.a[u]);
             const float2 drz = pmul(psub(ez_i.a[u], e.z.a[u]), c_dr), df = psub(ep_i.a[u], e.p.a[u]), sf = padd(ep_i.a[u], e.p.a[u]);
-            const float2 dr = pmul(dzr, c_dz);
-            tr[u] = pmul(dzp, c_dtdz);
-            tp[u] = psub(drz, dr);
+            tr[u] = pmul(dzp, c_ndz);                  // the curl; dt joins it in the last fma
+            tp[u] = pfma(dzr, c_ndz, drz);
             tz[u] = pfma(sf, hC, pmul(df, c_dr));
             if (zs && (unsigned)i < (unsigned)nr) {
                 const float2 b = both(__ldg(p.t.bz_h + k + u)), c = both(__ldg(p.t.cz_h + k + u));
-                const float2 v = pfma(zq[u], b, pmul(pmul(dzp, c_dz), c)), w = pfma(zq[zstr + u], b, pmul(dr, c));
-                tr[u] = pfma(v, c_dt, tr[u]);
+                const float2 v = pfma(zq[u], b, pmul(pmul(dzp, c_dz), c)), w = pfma(zq[zstr + u], b, pmul(pmul(dzr, c_dz), c));
+                tr[u] = psub(tr[u], v);
                 tp[u] = psub(tp[u], w);
                 if (level == 0) {
                     zq[u] = v;
@@ -287,9 +287,9 @@ __global__ void __launch_bounds__(NT, NT > 192 ? 1 : 2) k_two(const __grid_const
         for (int u = 0; u < 2; ++u) {
             tr[u] = pfma(psub(ez_j.a[u], e.z.a[u]), hA, tr[u]);
             tz[u] = pfma(psub(er_j.a[u], e.r.a[u]), hB, tz[u]);
-            h.r.a[u] = padd(h.r.a[u], tr[u]);
+            h.r.a[u] = pfma(tr[u], c_ndt, h.r.a[u]);
             h.p.a[u] = pfma(tp[u], c_dt, h.p.a[u]);
-            h.z.a[u] = psub(h.z.a[u], pmul(tz[u], c_dt));
+            h.z.a[u] = pfma(tz[u], c_ndt, h.z.a[u]);
         }
     };
     // E of the pair at radius i (0 <= i < n_r).  h: H there, hp_i, hz_i: one radius in, H: this thread's place
@@ -307,18 +307,19 @@ __global__ void __launch_bounds__(NT, NT > 192 ? 1 : 2) k_two(const __grid_const
         float2 tr[2], tp[2], tz[2], dzp[2], dzr[2];
 #pragma unroll
         for (int u = 0; u < 2; ++u) {
-            dzp[u] = pmul(psub(h.p.a[u], u ? h.p.a[0] : hp_k), c_dz);
-            dzr[u] = pmul(psub(h.r.a[u], u ? h.r.a[0] : hr_k), c_dz);
-            const float2 drz = pmul(psub(h.z.a[u], hz_i.a[u]), c_dr);
+            dzp[u] = psub(h.p.a[u], u ? h.p.a[0] : hp_k);
+            dzr[u] = psub(h.r.a[u], u ? h.r.a[0] : hr_k);
+            const float2 drz = pmul(psub(hz_i.a[u], h.z.a[u]), c_dr);          // minus d H_z / dr
             const float2 df = psub(h.p.a[u], hp_i.a[u]), sf = padd(h.p.a[u], hp_i.a[u]);
-            tp[u] = psub(dzr[u], drz);
+            tp[u] = pfma(dzr[u], c_dz, drz);
             tz[u] = pfma(sf, eC, pmul(df, c_dr));
             if (rslab(i) && live) {
                 const uint32_t rx = rx_at(i) + u;
                 float2 *rq = rbuf + ((i & 1) * 4 + 2) * SLAB + u;
-                const float2 br = both(__ldg(p.t.br_n + i)), cr = both(__ldg(p.t.cr_n + i));
+                const float2 br = both(__ldg(p.t.br_n + i));
+                const float cr = __ldg(p.t.cr_n + i);
                 const float2 a0 = level ? rq[0] : q.iP[PS_EP_R][rx], a1 = level ? rq[SLAB] : q.iP[PS_EZ_R][rx];
-                const float2 v = pfma(a0, br, pmul(drz, cr)), w = pfma(a1, br, pmul(tz[u], cr));
+                const float2 v = pfma(a0, br, pmul(drz, both(-cr))), w = pfma(a1, br, pmul(tz[u], both(cr)));
                 tp[u] = psub(tp[u], v);
                 tz[u] = padd(tz[u], w);
                 if (level == 0) {
@@ -329,7 +330,7 @@ __global__ void __launch_bounds__(NT, NT > 192 ? 1 : 2) k_two(const __grid_const
                     q.oP[PS_EZ_R][rx] = w;
                 }
             }
-            tr[u] = psub(pmul(psub(h.z.a[u], hz_j.a[u]), eA), dzp[u]);
+            tr[u] = pfma(psub(h.z.a[u], hz_j.a[u]), eA, pmul(dzp[u], c_ndz));
             tz[u] = pfma(psub(h.r.a[u], hr_j.a[u]), eB, tz[u]);
         }
         float cr_[2] = {cn[0], cn[1]}, cp_[2] = {cn[0], cn[1]}, cz_[2] = {cc[0], cc[1]};
@@ -338,7 +339,8 @@ __global__ void __launch_bounds__(NT, NT > 192 ? 1 : 2) k_two(const __grid_const
 #pragma unroll
                 for (int u = 0; u < 2; ++u) {
                     const float2 b = both(__ldg(p.t.bz_n + k + u)), c = both(__ldg(p.t.cz_n + k + u));
-                    const float2 v = pfma(zq[2 * zstr + u], b, pmul(dzp[u], c)), w = pfma(zq[3 * zstr + u], b, pmul(dzr[u], c));
+                    const float2 v = pfma(zq[2 * zstr + u], b, pmul(pmul(dzp[u], c_dz), c));
+                    const float2 w = pfma(zq[3 * zstr + u], b, pmul(pmul(dzr[u], c_dz), c));
                     tr[u] = psub(tr[u], v);
                     tp[u] = padd(tp[u], w);
                     if (level == 0) {

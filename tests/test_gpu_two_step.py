@@ -160,3 +160,22 @@ def test_a_timeout_under_the_decay_probe_is_reported_by_the_lens(use_graph):
     z.set_energy_probe(50)
     z.set_wait_limit(1 << 22)
     assert _rel(lens.forward([rho]), S) < 1e-5
+
+
+@pytest.mark.parametrize("name", ["cut_wedge", "whole_wedge", "wide_slabs", "no_slabs"])
+def test_two_step_errors_are_the_split_steps(name):
+    """An update adds its curl to the field in one rounding, as in the split step, so the errors against 64 bits are
+    those of another summation order of the same terms: within a quarter of each other."""
+    spec = _spec(name)
+    rho = smoothed_rho(spec.n_r_design, spec.n_phi, 5, mode="minmax")
+    _, g_ref, fwd, _ = O.gradient(spec, rho)
+    errs = []
+    for kernel in ((6, 16, 0), (0, 4, 0)):
+        z = _zone(spec, *kernel)
+        S = z.forward(_dev(rho))
+        des = np.moveaxis(z.design_dft(0).cpu().numpy(), 4, 2)
+        errs.append((_rel(des, fwd["des"]), _rel(z.monitor_dft().cpu().numpy(), fwd["mon"]),
+                     _rel(z.adjoint(4.0 * S).cpu().numpy(), g_ref)))
+    print(name, errs)
+    for two, split in zip(*errs):
+        assert two < 1.25 * split
