@@ -286,7 +286,7 @@ __global__ void __launch_bounds__(C == 1 ? RES_THREADS_1 : RES_THREADS, 1) k_res
         const int i = max(i0 - 1 + t, 0);
         float *r = itab + t * ITAB;
         const float irn = p.t.inv_r_n[i], irh = p.t.inv_r_h[i];
-        r[T_HA] = -dt * irn * dphi1; r[T_HB] = -irh * dphi1; r[T_HC] = 0.5f * irh;
+        r[T_HA] = irn * dphi1; r[T_HB] = -irh * dphi1; r[T_HC] = 0.5f * irh;
         r[T_EA] = irh * dphi1; r[T_EB] = -irn * dphi1; r[T_EC] = 0.5f * irn;
         r[T_BRN] = p.t.br_n[i]; r[T_CRN] = p.t.cr_n[i];
         r[T_BRH] = p.t.br_h[i]; r[T_CRH] = p.t.cr_h[i];
@@ -497,7 +497,7 @@ __global__ void __launch_bounds__(C == 1 ? RES_THREADS_1 : RES_THREADS, 1) k_res
     fa.ncd = ncd; fa.nd = nd; fa.rows = rows; fa.nj = nj; fa.i0 = i0; fa.j0 = j0; fa.d0 = d0;
     fa.h_des = h_des; fa.h_mon = h_mon;
     const float2 c_dz = both(p.inv_dz), c_ndz = both(-p.inv_dz), c_dr = both(p.inv_dr);
-    const float2 c_dt = both(dt), c_ndt = both(-dt), c_dtdz = both(dt * p.inv_dz);
+    const float2 c_dt = both(dt), c_ndt = both(-dt);
     const float2 *E1 = E + NX, *E2 = E + 2 * NX, *H1 = H + NX, *H2 = H + 2 * NX;
     __syncthreads();
 
@@ -522,8 +522,8 @@ __global__ void __launch_bounds__(C == 1 ? RES_THREADS_1 : RES_THREADS, 1) k_res
         const float2 ep_i = E1[o + SI];
         const float2 dzp = psub(E1[o + 1], ep), dzr = psub(E[o + 1], er), drz = psub(E2[o + SI], ez);
         const float2 df = psub(ep_i, ep), sf = padd(ep_i, ep);
-        float2 tr = pmul(dzp, c_dtdz);                       // dt times the curl of H_r
-        float2 tp = pfma(dzr, c_ndz, pmul(drz, c_dr));       // curls of H_phi, of H_z
+        float2 tr = pmul(dzp, c_ndz);                        // curls of H_r, of H_phi, of H_z; dt joins them in the last fma
+        float2 tp = pfma(dzr, c_ndz, pmul(drz, c_dr));
         float2 tz = pfma(sf, both(it[T_HC]), pmul(df, c_dr));
         const uint32_t pz = psi & 0xffffu, pr = psi >> 16;
         if (pz != NO_PSI) {
@@ -533,7 +533,7 @@ __global__ void __launch_bounds__(C == 1 ? RES_THREADS_1 : RES_THREADS, 1) k_res
             const float2 v = pfma(pzH[pzHs + pz], bz, pmul(pmul(dzr, c_dz), cz));
             pzH[pz] = u;
             pzH[pzHs + pz] = v;
-            tr = pfma(u, c_dt, tr);
+            tr = psub(tr, u);
             tp = psub(tp, v);
         }
         if (pr != NO_PSI) {
@@ -548,7 +548,7 @@ __global__ void __launch_bounds__(C == 1 ? RES_THREADS_1 : RES_THREADS, 1) k_res
                 const float2 X = pmul(gz, both(dphi1));
                 const float2 m = pfma(pmH[pr], both(it[T_BMN]), pmul(X, both(it[T_CMN])));
                 pmH[pr] = m;
-                tr = pfma(padd(X, m), both(-dt * it[T_IRN]), tr);
+                tr = pfma(padd(X, m), both(it[T_IRN]), tr);
                 const float2 Y = pfma(sf, both(0.5f), pmul(gr, both(-dphi1)));
                 const float2 mz = pfma(pmH[prHs + pr], both(it[T_BMH]), pmul(Y, both(it[T_CMH])));
                 pmH[prHs + pr] = mz;
@@ -563,7 +563,7 @@ __global__ void __launch_bounds__(C == 1 ? RES_THREADS_1 : RES_THREADS, 1) k_res
             tr = pfma(gz, both(it[T_HA]), tr);
             tz = pfma(gr, both(it[T_HB]), tz);
         }
-        H[o] = hr = padd(hr, tr);
+        H[o] = hr = pfma(tr, c_ndt, hr);
         H[NX + o] = hp = pfma(tp, c_dt, hp);
         H[2 * NX + o] = hz = pfma(tz, c_ndt, hz);
     };

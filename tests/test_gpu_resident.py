@@ -210,3 +210,25 @@ def test_a_run_that_gives_up_waiting_is_repeated_by_the_split_step(name):
     a.set_wait_limit(1 << 22)
     n0 = a.launches
     assert np.array_equal(a.forward(rho), want) and a.launches - n0 < 20
+
+
+@pytest.mark.parametrize("form", [0, 1])
+@pytest.mark.parametrize("name", ["tiny", "odd", "two_cells", "axis"])
+def test_one_launch_errors_are_the_split_steps(name, form):
+    """The coefficients of an update are rounded as often as the split step's, so the errors against 64 bits are those
+    of another summation order of the same terms: within a quarter of each other."""
+    spec = _spec(name)
+    rho = _rho(spec)
+    _, g_ref, fwd, _ = O.gradient(spec, rho, pml_form=form)
+    errs = []
+    for split in (False, True):
+        z = _zone(spec, form)
+        if split:
+            z.set_kernel(0, 4, 0)
+        S = z.forward(_dev(rho))
+        des = np.moveaxis(z.design_dft(0).cpu().numpy(), 4, 2)
+        errs.append((_rel(des, fwd["des"]), _rel(z.monitor_dft().cpu().numpy(), fwd["mon"]),
+                     _rel(z.adjoint(4.0 * S).cpu().numpy(), g_ref)))
+    print(name, form, errs)
+    for one, split in zip(*errs):
+        assert one < 1.25 * split
