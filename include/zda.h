@@ -240,7 +240,8 @@ long long zda_zone_launch_count(const zda_zone *zone);
  * in {4, 8, 16} phi rows streaming over one of i_ranges radius ranges (0 =
  * by a cost rule), ping-pong buffers; a run under the decay probe takes the
  * split step.  Default at zone creation: variant 6 with 16 rows where it
- * applies and the zone has at least 2.2 million cells and 128 radii; else
+ * applies, the zone has at least 2.2 million cells and 128 radii and its
+ * plan's estimate is below the split step's time (all but flat zones); else
  * variant 4 with 16 rows where it applies and the zone gives at least four
  * waves of its thread blocks (2 per SM) in radius ranges of about 21 radii;
  * else variant 0.  A zone with the default variant 0 whose whole field state

@@ -911,6 +911,21 @@ static zda::TwoPlan two_step_plan(const zda_zone &z)
     return zda::two_plan(p, z.tile_phi, std::min(z.i_ranges, z.d.n_r), sms, (size_t)smem);
 }
 
+// Whether a default zone takes two steps per launch (on tiles of 16 phi rows): from 2.2 M cells on, if there are 128
+// radii to stream over and the plan's estimate is below what the split step takes: tiles short in z hold few cells and
+// much z-PML.  Measured on GB300 over 110 zones of 2.2 to 9 M cells; us per step of a forward and adjoint run, two-step |
+// split, by the estimate per cell: 0.027 2000 x 11 x 112 cells 74 | 92; 0.030 252 x 201 x 134 195 | 237; 0.033 181 x 107 x
+// 160 91 | 99; 0.036 262 x 136 x 100 124 | 137; 0.038 160 x 200 x 100 129 | 122, 209 x 143 x 104 104 | 114; 0.039 129 x 233 x
+// 90 101 | 97; past the line 0.042 304 x 305 x 60 197 | 188; 0.044 290 x 136 x 60 97 | 85; 0.047 130 x 330 x 60 112 | 93.
+// Below 2.2 M cells the split step wins earlier: 208 x 48 x 160 56 | 44, 333 x 48 x 100 60 | 57; 60 x 320 x 160 107 | 99.
+static bool takes_two_steps(const zda_zone &z)
+{
+    const double cells = (double)z.d.n_r * z.d.n_phi * z.d.n_z;
+    if (z.d.n_fold == 0 || z.d.n_r < 128 || cells < 2.2e6) return false;
+    const zda::TwoPlan pl = two_step_plan(z);
+    return pl.ranges && pl.cost < 0.0395 * cells;
+}
+
 // Whether the split step of a default zone runs its E update on TMA tiles of 16 phi rows: annular, even n_z
 // and z-PML, and at least four waves of thread blocks (2 per SM) in radius ranges of about 21 radii.  Slower
 // on zones of 16 or fewer phi cells and on the 200-phi-cell zones of the 40-zone lens, where ranges get short.
@@ -1348,19 +1363,10 @@ zda_status zda_zone_create(zda_ctx *ctx, const zda_zone_desc *desc, zda_zone **o
     zda_zone *z = new zda_zone();
     z->ctx = ctx;
     z->d = *desc;
-    // default step, on zones too large for the resident step (annular, even n_z and z-PML).  Two steps per
-    // launch on tiles of 16 phi rows from 2.2 M cells on, if there are 128 radii to stream over; else the
-    // split step (split_takes_tiles).  Measured on GB300, us per step, two-step | split (the
-    // better of its forms): 300 x 320 x 160 cells 330 | 391; 144 x 128 x 160 81 | 93; 157 x 96 x 160 62 | 77;
-    // 216 x 114 x 112 84 | 94; below the line 208 x 48 x 160 49 | 44; 123 x 95 x 62 33 | 25; 916 x 16 x 100
-    // 48 | 43; and with few radii 60 x 320 x 160 107 | 99.
-    if (desc->n_fold > 0 && desc->n_r >= 128 && (double)desc->n_r * desc->n_phi * desc->n_z >= 2.2e6) {
-        z->variant = 6;
-        z->tile_phi = 16;
-        if (!two_step_plan(*z).ranges) z->variant = 0;
-    }
-    if (z->variant == 0 && split_takes_tiles(*desc)) z->variant = 4;
-    z->tile_phi = z->variant ? 16 : 2;
+    // default step, on zones too large for the resident step
+    z->tile_phi = 16;
+    z->variant = takes_two_steps(*z) ? 6 : split_takes_tiles(*desc) ? 4 : 0;
+    if (!z->variant) z->tile_phi = 2;
     zda_status st = derive(*z);
     if (st != ZDA_OK) { delete z; return st; }
     *out = z;

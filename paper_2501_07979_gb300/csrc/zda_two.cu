@@ -512,15 +512,17 @@ TwoPlan two_plan(const StepParams &p, int rows, int ranges, int sms, size_t smem
             const int occ = std::max(1, std::min((int)((smem_limit + 1024) / (L.bytes + 1024)), 65536 / (168 * nt)));
             const long long blocks = (long long)tiles_j * tiles_k * ((p.nr + len - 1) / len);
             // blocks differ (slabs, design layer): more than one wave of them queues up with half a block to
-            // spare, a single wave waits for its slowest (300 x 320 x 160 cells, us per step with DFTs at 3 to 10
-            // ranges: 399, 383, 393, 366 at 6, 380 at 8; 144 x 128 x 160: 93 at 3, 113 at 2, 98 at 6)
+            // spare, a single wave waits for its slowest (144 x 128 x 160 cells, us per step of a run at 1 to 6 ranges:
+            // 187, 115, 93, 117, 107, 98)
             const double slots = (double)sms * occ, waves = blocks <= slots ? 1.2 : blocks / slots + 0.6;
-            // a radius costs a thread's latency or its share of the SM, whichever is longer
-            const double per_radius = std::max(1100.0, 4.2 * occ * t.threads());
+            // a radius costs its serial chain and little for each thread more (over 120 zones 2.8 us at 288 threads,
+            // 3.0 at 384), and longer the more of the z-pairs lie in the PML (3.0 us at a tenth, 3.8 at a quarter)
+            const double per_radius = (950.0 + 1.22 * occ * t.threads()) * (1.0 + 1.8 * 2 * p.pz / p.nz);
             const double cost = waves * (len + 5.0) * per_radius;
             if (cost < best_cost) {
                 best_cost = cost;
                 best = t;
+                best.cost = cost;
                 best.ranges = (p.nr + len - 1) / len;
                 best.smem = (size_t)L.bytes;
             }

@@ -13,6 +13,7 @@ struct TwoPlan {
     int nrow = 0, npair = 0;           // rows and z-pairs of a tile with its halo: one thread each
     int nzq = 0;                       // most z-pairs of a tile that lie in the z-PML
     size_t smem = 0;
+    double cost = 0;                   // estimate of a launch's time, in units of about 1.8 ns
     int threads() const { return (nrow * npair + 31) / 32 * 32; }
 };
 

@@ -163,3 +163,26 @@ def test_evaluation_calls_check_their_arguments_before_any_device_work(libpath):
     assert L.zda_field_intensity(None, 1, 1, 1.0, None, None) == _lib.ERR_ARG
     assert L.zda_encircled_power(None, None, 1, 0, None, None) == _lib.ERR_ARG
     assert b"bad argument" in L.zda_last_error() or b"null" in L.zda_last_error()
+
+
+@pytest.mark.parametrize("shape,two_steps", [
+    ((2000, 11, 112), True), ((1500, 16, 100), True), ((144, 128, 160), True), ((300, 320, 160), True), ((208, 291, 66), True),
+    ((130, 330, 52), False), ((290, 136, 60), False), ((190, 162, 78), False), ((304, 305, 60), False),   # flat: slower by it
+    ((208, 48, 160), False), ((100, 320, 160), False), ((300, 320, 159), False)])      # small, few radii, odd n_z
+def test_default_step_is_the_faster_one(libpath, shape, two_steps):
+    """Which large zones take two steps per launch, on both sides of the line (times beside the rule)."""
+    from paper_2501_07979_gb300 import _lib
+    from paper_2501_07979_gb300.zone import make_desc
+    from zda_inputs import zone_tiny
+    L = _lib.load(libpath)
+    nr, nphi, nz = shape
+    k0 = nz // 3
+    spec = zone_tiny(n_r=nr, n_phi=nphi, n_z=nz, n_fold=400, r_lo=200.0, dr=0.05, dz=0.05, pml_r_in=8, pml_r_out=8, pml_z=8,
+                     layer_k0=(0, k0, k0 + 5), design_k0=k0, design_k1=k0 + 5, monitor_k=nz - 12, source_k=10, filter_radius=0.1)
+    ctx = ctypes.create_string_buffer(64)         # zone creation only stores the context pointer
+    h = ctypes.c_void_p()
+    assert L.zda_zone_create(ctx, ctypes.byref(make_desc(spec)), ctypes.byref(h)) == _lib.OK
+    v, t, r = ctypes.c_int(), ctypes.c_int(), ctypes.c_int()
+    assert L.zda_zone_get_kernel(h, ctypes.byref(v), ctypes.byref(t), ctypes.byref(r)) == _lib.OK
+    L.zda_zone_destroy(h)
+    assert (v.value == 6) == two_steps
