@@ -256,6 +256,9 @@ long long zda_zone_launch_count(const zda_zone *zone);
  * to 5 and the one-launch run bound their device-side waits
  * (zda_zone_set_wait_limit). */
 zda_status zda_zone_set_kernel(zda_zone *zone, int variant, int tile_phi, int i_ranges);
+/* Takes the choice back: the default above for the zone's r-PML form, the
+ * one-launch run of a small zone included (no zda_zone_set_kernel gives that). */
+zda_status zda_zone_default_kernel(zda_zone *zone);
 zda_status zda_zone_get_kernel(const zda_zone *zone, int *variant, int *tile_phi, int *i_ranges);
 
 /* Form of the radial PML ("Differentiable FDTD in cylindrical coordinates":

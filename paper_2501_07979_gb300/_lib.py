@@ -76,6 +76,7 @@ SIGNATURES = {
     "zda_copy_design_dft": (_i, [_vp, _i, _vp, _vp]),
     "zda_zone_launch_count": (ctypes.c_longlong, [_vp]),
     "zda_zone_set_kernel": (_i, [_vp, _i, _i, _i]),
+    "zda_zone_default_kernel": (_i, [_vp]),
     "zda_zone_get_kernel": (_i, [_vp, ctypes.POINTER(_i), ctypes.POINTER(_i), ctypes.POINTER(_i)]),
     "zda_zone_set_radial_pml": (_i, [_vp, _i]),
     "zda_zone_get_radial_pml": (_i, [_vp, ctypes.POINTER(_i)]),

@@ -942,6 +942,16 @@ static bool split_takes_tiles(const zda_zone_desc &d)
     return tiles * (d.n_r / 21) >= 8LL * sms;
 }
 
+// The step of a zone whose caller chose none: by size, and of zones too large for the resident step.
+static void choose_default(zda_zone &z)
+{
+    z.kernel_default = z.pair_kernels = true;
+    z.i_ranges = 0;
+    z.tile_phi = 16;
+    z.variant = z.rpml ? 0 : takes_two_steps(z) ? 6 : split_takes_tiles(z.d) ? 4 : 0;
+    if (!z.variant) z.tile_phi = 2;
+}
+
 // A run by the two-step form: state and CPML auxiliaries change buffers with
 // every launch; a last odd step is a split step on the buffer it finds.
 static zda_status two_step_loop(zda_zone &z, zda::StepParams &p, cudaStream_t s)
@@ -1363,10 +1373,7 @@ zda_status zda_zone_create(zda_ctx *ctx, const zda_zone_desc *desc, zda_zone **o
     zda_zone *z = new zda_zone();
     z->ctx = ctx;
     z->d = *desc;
-    // default step, on zones too large for the resident step
-    z->tile_phi = 16;
-    z->variant = takes_two_steps(*z) ? 6 : split_takes_tiles(*desc) ? 4 : 0;
-    if (!z->variant) z->tile_phi = 2;
+    choose_default(*z);
     zda_status st = derive(*z);
     if (st != ZDA_OK) { delete z; return st; }
     *out = z;
@@ -1622,10 +1629,8 @@ zda_status zda_copy_design_dft(zda_zone *z, int which, float *out, void *stream)
 
 long long zda_zone_launch_count(const zda_zone *z) { return z ? z->launches : -1; }
 
-zda_status zda_zone_set_kernel(zda_zone *z, int variant, int tile_phi, int i_ranges)
+static zda_status set_kernel(zda_zone *z, int variant, int tile_phi, int i_ranges)
 {
-    if (!z || variant < 0 || variant > 6 || i_ranges < 0) return fail(ZDA_ERR_ARG, "bad kernel choice");
-    z->kernel_default = false;
     if (variant == 6) {                      // two steps per launch on tiles streaming along r
         if (z->d.n_fold == 0) return fail(ZDA_ERR_ARG, "the axis zone (continuous axisymmetry) uses the split step");
         if (z->rpml) return fail(ZDA_ERR_ARG, "the two-step form implements the real-radius r-PML only");
@@ -1688,6 +1693,22 @@ zda_status zda_zone_set_kernel(zda_zone *z, int variant, int tile_phi, int i_ran
     z->variant = variant;
     z->tile_phi = tile_phi;
     z->i_ranges = i_ranges;
+    z->have_forward = false;
+    return ZDA_OK;
+}
+
+zda_status zda_zone_set_kernel(zda_zone *z, int variant, int tile_phi, int i_ranges)
+{
+    if (!z || variant < 0 || variant > 6 || i_ranges < 0) return fail(ZDA_ERR_ARG, "bad kernel choice");
+    const zda_status st = set_kernel(z, variant, tile_phi, i_ranges);
+    if (st == ZDA_OK) z->kernel_default = false;
+    return st;
+}
+
+zda_status zda_zone_default_kernel(zda_zone *z)
+{
+    if (!z) return fail(ZDA_ERR_ARG, "null zone");
+    choose_default(*z);
     z->have_forward = false;
     return ZDA_OK;
 }

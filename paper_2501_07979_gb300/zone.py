@@ -209,6 +209,11 @@ class Zone:
         tile; i_ranges radius ranges)."""
         check(_lib.lib().zda_zone_set_kernel(self.handle, int(variant), int(tile_phi), int(i_ranges)))
 
+    def default_kernel(self):
+        """Takes set_kernel back: the kernel the library chose at creation, or
+        the one-launch run of a small zone, which set_kernel cannot choose."""
+        check(_lib.lib().zda_zone_default_kernel(self.handle))
+
     def set_radial_pml(self, form):
         """r-PML form: 0 convolutional PML with the real radius (default),
         1 stretched coordinates (split radial curl, stretched outer radius)."""

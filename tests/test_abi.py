@@ -186,3 +186,8 @@ def test_default_step_is_the_faster_one(libpath, shape, two_steps):
     assert L.zda_zone_get_kernel(h, ctypes.byref(v), ctypes.byref(t), ctypes.byref(r)) == _lib.OK
     L.zda_zone_destroy(h)
     assert (v.value == 6) == two_steps
+
+
+def test_default_kernel_refuses_a_missing_zone(libpath):
+    from paper_2501_07979_gb300 import _lib
+    assert _lib.load(libpath).zda_zone_default_kernel(None) == _lib.ERR_ARG

@@ -232,3 +232,46 @@ def test_one_launch_errors_are_the_split_steps(name, form):
     print(name, form, errs)
     for one, split in zip(*errs):
         assert one < 1.25 * split
+
+
+def test_the_default_comes_back():
+    """A refused choice leaves the one-launch run, a made one ends it, and the default brings it back."""
+    from paper_2501_07979_gb300 import ZdaError
+    spec = _spec("tiny")
+    z = _zone(spec)
+    r = _dev(_rho(spec))
+
+    def launches():
+        n0 = z.launches
+        z.forward(r)
+        return z.launches - n0
+
+    assert launches() < 20
+    for bad in ((1, 3, 0), (3, 5, 0), (4, 4, 0), (6, 5, 0), (7, 16, 0), (0, 4, -1)):
+        with pytest.raises(ZdaError, match="ZDA_ERR_ARG"):
+            z.set_kernel(*bad)
+    assert launches() < 20
+    z.set_kernel(0, 4, 0)
+    assert launches() >= 2 * spec.n_steps
+    z.default_kernel()
+    assert z.get_kernel() == (0, 2, 0) and launches() < 20
+    z.set_kernel(2, 2, 0)
+    z.set_radial_pml(1)
+    z.default_kernel()
+    assert launches() < 20
+
+
+@pytest.mark.parametrize("name", ["tiny", "axis"])
+def test_a_tuned_small_zone_keeps_its_one_launch_run(tmp_path, name):
+    from paper_2501_07979_gb300.autotune import candidates, tune_zone
+    spec = _spec(name)
+    cache = str(tmp_path / "tiles.json")
+    z = _zone(spec)
+    choice, times = tune_zone(z, cache_path=cache)
+    assert set(times) - set(candidates(spec)) == {(0, 2, 0)} and times[choice] == min(times.values())
+    z2 = _zone(spec)
+    assert tune_zone(z2, cache_path=cache) == (choice, {})
+    for t in (z, z2):
+        n0 = t.launches
+        t.forward(_dev(_rho(spec)))
+        assert choice == (0, 2, 0) and t.launches - n0 < 20
