@@ -250,7 +250,8 @@ static void compute_layout(zda_zone &z)
     // second field buffer and CPML sets for the fused and two-step (ping-pong) forms
     L.fields2 = take(6 * ncell * sizeof(float2));
     L.psi_h2 = take((2 * plane * 2 * d.pml_z + 2 * (size_t)(d.pml_r_in + d.pml_r_out) * np * nz) * sizeof(float2));
-    L.psi_e2 = take((2 * plane * 2 * d.pml_z + 2 * (size_t)(d.pml_r_in + d.pml_r_out) * np * nz) * sizeof(float2));
+    const bool two = d.n_fold > 0 && d.n_z % 2 == 0 && d.pml_z % 2 == 0;      // only the two-step form needs the E side twice
+    L.psi_e2 = take(two ? (2 * plane * 2 * d.pml_z + 2 * (size_t)(d.pml_r_in + d.pml_r_out) * np * nz) * sizeof(float2) : 0);
     L.mon = take(Q * 2 * plane * sizeof(float2));
     L.des_f = take(Q * 3 * plane * z.nk * sizeof(float2));
     L.des_a = take(Q * 3 * plane * z.nk * sizeof(float2));

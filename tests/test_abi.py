@@ -191,3 +191,25 @@ def test_default_step_is_the_faster_one(libpath, shape, two_steps):
 def test_default_kernel_refuses_a_missing_zone(libpath):
     from paper_2501_07979_gb300 import _lib
     assert _lib.load(libpath).zda_zone_default_kernel(None) == _lib.ERR_ARG
+
+
+def test_only_two_step_zones_pay_for_its_second_auxiliaries(libpath):
+    """The workspace grows by linear terms in n_z (the coefficient tables, fields, slabs); the second set of E-side
+    CPML auxiliaries is there at even n_z only, where the two-step form can run."""
+    from paper_2501_07979_gb300 import _lib
+    from paper_2501_07979_gb300.zone import make_desc
+    from zda_inputs import zone_tiny
+    L = _lib.load(libpath)
+    ctx = ctypes.create_string_buffer(64)         # zone creation only stores the context pointer
+
+    def bytes_of(**kw):
+        spec = zone_tiny(n_r=64, n_phi=96, n_fold=20, **kw)
+        h, n = ctypes.c_void_p(), ctypes.c_size_t()
+        assert L.zda_zone_create(ctx, ctypes.byref(make_desc(spec)), ctypes.byref(h)) == _lib.OK
+        assert L.zda_zone_workspace_bytes(h, ctypes.byref(n)) == _lib.OK
+        L.zda_zone_destroy(h)
+        return n.value, spec
+
+    (lo, _), (mid, s), (hi, _) = (bytes_of(n_z=k) for k in (60, 61, 62))
+    psi = 8 * 2 * s.n_phi * (s.n_r * 2 * s.pml_z + (s.pml_r_in + s.pml_r_out) * s.n_z)
+    assert abs((lo + hi) / 2 - mid - psi) < 64 * 256                   # each array is rounded up to 256 bytes
