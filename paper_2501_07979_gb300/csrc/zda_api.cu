@@ -1468,12 +1468,13 @@ zda_status zda_filter_project_backward(zda_zone *z, const float *rho, const floa
     return ZDA_OK;
 }
 
-// Whether the fields that a forward run ends with may have decayed to the run's rounding noise.  There two forms of
-// the step agree with the exact fields equally well but not with each other, so a run whose final fields the caller
-// may read keeps the split step's.  Over 1432 random zones the resident step's final fields were 2e-5 to 6e-4 away
-// from the split step's on 82 (the exact ones 3e-5 from both): all with cells of less than 0.03 wavelengths, or with
-// at most 1.5 wavelengths between the PMLs at cells of 0.05, none at 0.1; at the sizes let through at most 1e-5.
-// The monitor DFTs differ by at most 1.5e-6 on all of them.
+// Whether the fields that a forward run ends with may have decayed far below their peak.  There two forms of the step
+// are equally far from the exact fields but not on the same side of them, so a run whose final fields the caller may
+// read keeps the split step's.  Over 1432 random zones of 6.5 to 9 time units the one-launch run's final fields were 2e-5
+// to 6e-4 away from the split step's on 82: all with cells of less than 0.03 wavelengths, or with at most 1.5 wavelengths
+// between the PMLs at cells of 0.05, none at 0.1; at the sizes let through at most 1e-5, and the monitor DFTs at most
+// 1.5e-6 on all of them.  Against 64 bits (24 x 8 x 40 cells): at 0.03, kept from the one-launch run, every form of the
+// step is 8e-5 to 1e-4 off, the split step too; at 0.1 both 2e-6 after 6.5 time units, 1.1e-5 after 40 and 3e-5 after 100.
 static bool final_fields_decay(const zda_zone &z)
 {
     const zda_zone_desc &d = z.d;
