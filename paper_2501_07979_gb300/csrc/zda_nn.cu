@@ -593,8 +593,9 @@ zda_status layer_grad(zda_nn *net, int li, int n, const uint16_t *x0, const uint
     const Layer &l = net->L[li];
     const long P = pos_count(net, l.level, n), rows = net->rows[l.level];
     const int Wp = net->W[l.level] + 2, taps = l.k * l.k;
-    // all 3x3 layers but the first have 64 channels per tensor and fit the one-window kernel
-    const bool win = taps == 9 && l.cin_pad % C == 0 && ldg == C && Wp + 1 <= WW_MAX_HALO;
+    // all 3x3 layers but the first have 64 channels per tensor and take the one-window kernel
+    static_assert(176 + 2 + 1 <= WW_MAX_HALO, "a window of the widest image fits its seven chunks");
+    const bool win = taps == 9 && l.cin_pad % C == 0;
     int splits, ngroups = 0, ntap_grp = 0, nrow;
     cudaError_t e;
     if (win) {
@@ -626,7 +627,6 @@ zda_status layer_grad(zda_nn *net, int li, int n, const uint16_t *x0, const uint
         p.cin_planes = l.cin_pad / 8;
         p.ntap_grp = ntap_grp = 16 / p.cin_planes;
         p.ngroups = ngroups = (p.taps + p.ntap_grp - 1) / p.ntap_grp;
-        p.two_inputs = x1 != nullptr;
         p.N = ldg;
         p.kt = WG_KT;
         p.ntiles = (p.P + p.kt - 1) / p.kt;
@@ -637,8 +637,7 @@ zda_status layer_grad(zda_nn *net, int li, int n, const uint16_t *x0, const uint
         if ((size_t)splits * nrow * p.N > net->wpart_floats)
             return nn_fail(ZDA_ERR_OOM, "weight-gradient partial buffer too small");
         p.rows = rows;
-        p.x0 = x0;
-        p.x1 = x1;
+        p.x = x0;
         p.dy = g;
         p.partial = at<float>(net, net->o.wpart);
         p.err = at<int>(net, net->o.err);

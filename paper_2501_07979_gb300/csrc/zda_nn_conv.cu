@@ -12,9 +12,12 @@
 //               each side) serves all taps: tap t is the same window seen
 //               from start row halo + off(t), i.e. a different descriptor
 //               start address, so no im2col copy is ever made.
-// k_wgrad_tc -- weight gradient: both operands MN-major (channels contiguous),
-//               reduction over positions; M = 128 rows hold 128 / c_in taps'
-//               shifted copies of the input, each copied pre-shifted.
+// k_wgrad_tc -- weight gradient of the first layer and the head: both operands
+//               MN-major (channels contiguous), reduction over positions; M =
+//               128 rows hold 128 / c_in taps' shifted copies of the input,
+//               each copied pre-shifted.
+// k_wgrad_win -- weight and bias gradient of the other layers, all taps of a
+//               64-channel input from one window.
 //
 // Roles of k_conv_tc (608 threads): warp 0 lane 0 = producer, warps 1 and 10
 // lane 0 = MMA issuers (M tile 0 / 1 of each tile, warp 1 also allocates
@@ -436,13 +439,9 @@ __global__ void __launch_bounds__(WG_THREADS, 1)
                 int t = g * p.ntap_grp + j;
                 if (t >= p.taps) t = p.taps - 1;                 // padding copy: its rows are discarded
                 const int off = p.taps == 9 ? (t / 3 - 1) * p.Wp + (t % 3 - 1) : 0;
-                for (int c = 0; c < p.cin_planes; ++c) {
-                    const bool second = p.two_inputs && c >= 8;
-                    const uint16_t *x = second ? p.x1 : p.x0;
-                    const int cc = second ? c - 8 : c;
-                    bulk_load(sa + (j * p.cin_planes + c) * planeb, x + ((size_t)cc * p.rows + LEAD + y + off) * 8, planeb,
+                for (int c = 0; c < p.cin_planes; ++c)
+                    bulk_load(sa + (j * p.cin_planes + c) * planeb, p.x + ((size_t)c * p.rows + LEAD + y + off) * 8, planeb,
                               barF + 8 * s);
-                }
             }
             for (int c = 0; c < p.N / 8; ++c)
                 bulk_load(sb + c * planeb, p.dy + ((size_t)c * p.rows + LEAD + y) * 8, planeb, barF + 8 * s);

@@ -59,16 +59,15 @@ struct ConvParams {
 struct WgradParams {
     int P, Hp, Wp;
     int taps;              // 9 or 1
-    int cin_planes;        // input channels / 8 per tap copy (2, 4, 8 or 16)
+    int cin_planes;        // input channels / 8 per tap copy (2 or 8)
     int ntap_grp;          // taps per 128-row group (16 / cin_planes)
     int ngroups;           // ceil(taps / ntap_grp)
-    int two_inputs;        // planes 8..15 come from the second tensor (concatenated input)
     int N;                 // output channels (GEMM N)
     int kt;                // positions per stage (128)
     int ntiles;            // ceil(P / kt)
     int tiles_per_cta;
-    long rows;             // rows per plane of x0, x1 and dy
-    const uint16_t *x0, *x1, *dy;   // planar input(s) and output gradient
+    long rows;             // rows per plane of x and dy
+    const uint16_t *x, *dy;         // planar input and output gradient
     float *partial;        // [splits][ngroups][128][N]
     int *err;
     int wait_limit;
