@@ -3,18 +3,18 @@
 //
 // Why: a step of the split kernels moves 144 B per cell (each half reads six
 // components and writes three), one fused step 96 B, two fused steps 96 B for
-// both.  Measured per step (no source, no DFT): 300 x 320 x 160 cells 391 us by
-// the split step with its E half on TMA tiles, 330 here; 144 x 128 x 160 93 and
-// 81; 157 x 96 x 160 77 and 62.  With source, DFT history and its flush, per
-// step of a forward and adjoint run: 412 -> 390, 102 -> 93; a lens of five such
-// zones and the axis zone 404 -> 292 ms (with the axis zone's one-launch run).
+// both.  Measured per step (no source, no DFT): 300 x 320 x 160 cells 388 us by
+// the split step with its E half on TMA tiles, 323 here; 144 x 128 x 160 89 (by
+// pairs) and 81.  With source, DFT history and its flush, per step of a forward
+// and adjoint run: 412 -> 362, 102 -> 93; a lens of five such zones and the axis
+// zone (a split step in a lens) 404 -> 293 ms per iteration.
 //
-// What bounds it now: instructions and their latency, not memory (DRAM at 35 %
-// of its peak, shared memory at 45 %, 25 % of issue slots with 12 warps per SM;
-// without loads and stores the 300 x 320 x 160 zone would take 232 us).  Tried
-// and slower: one z-cell per thread at twice the warps (419 us: the extra
-// shared-memory instructions), the planes of a thread carried in registers
-// over the loop (361; with spills 1364).
+// What bounds it now: instructions and their latency, not memory (on the 300 x
+// 320 x 160 zone: DRAM at 33 % of its peak, shared memory at 38 %, 31 % of issue
+// slots with 12 warps per SM; without loads and stores it would take 232 of 330
+// us).  Tried and slower: one z-cell per thread at twice the warps (419 us: the
+// extra shared-memory instructions), the planes of a thread carried in
+// registers over the loop (361; with spills 1364).
 //
 // A thread block owns a tile of phi rows x z-cells and streams along r over a
 // range of radii; each thread holds one z-pair of one row of the tile or of
@@ -249,10 +249,10 @@ __global__ void __launch_bounds__(NT, NT > 192 ? 1 : 2) k_two(const __grid_const
 #pragma unroll
         for (int u = 0; u < 2; ++u) {
             const float2 dzp = psub(u ? ep_k : e.p.a[1], e.p.a[u]), dzr = psub(u ? er_k : e.r.a[1], e.r.a[u]);
-            const float2 drz = pmul(psub(ez_i.a[u], e.z.a[u]), c_dr), df = psub(ep_i.a[u], e.p.a[u]), sf = padd(ep_i.a[u], e.p.a[u]);
+            const float2 dr0 = psub(ez_i.a[u], e.z.a[u]), drz = pmul(dr0, c_dr), df = psub(ep_i.a[u], e.p.a[u]), sf = padd(ep_i.a[u], e.p.a[u]);
             tr[u] = pmul(dzp, c_ndz);                  // the curl; dt joins it in the last fma
-            tp[u] = pfma(dzr, c_ndz, drz);
-            tz[u] = pfma(sf, hC, pmul(df, c_dr));
+            tp[u] = pfma(dr0, c_dr, pmul(dzr, c_ndz));
+            tz[u] = pfma(df, c_dr, pmul(sf, hC));       // the small term is the one rounded
             if (zs && (unsigned)i < (unsigned)nr) {
                 const float2 b = both(__ldg(p.t.bz_h + k + u)), c = both(__ldg(p.t.cz_h + k + u));
                 const float2 v = pfma(zq[u], b, pmul(pmul(dzp, c_dz), c)), w = pfma(zq[zstr + u], b, pmul(pmul(dzr, c_dz), c));
@@ -309,10 +309,10 @@ __global__ void __launch_bounds__(NT, NT > 192 ? 1 : 2) k_two(const __grid_const
         for (int u = 0; u < 2; ++u) {
             dzp[u] = psub(h.p.a[u], u ? h.p.a[0] : hp_k);
             dzr[u] = psub(h.r.a[u], u ? h.r.a[0] : hr_k);
-            const float2 drz = pmul(psub(hz_i.a[u], h.z.a[u]), c_dr);          // minus d H_z / dr
+            const float2 dr0 = psub(hz_i.a[u], h.z.a[u]), drz = pmul(dr0, c_dr);          // minus d H_z / dr
             const float2 df = psub(h.p.a[u], hp_i.a[u]), sf = padd(h.p.a[u], hp_i.a[u]);
-            tp[u] = pfma(dzr[u], c_dz, drz);
-            tz[u] = pfma(sf, eC, pmul(df, c_dr));
+            tp[u] = pfma(dr0, c_dr, pmul(dzr[u], c_dz));
+            tz[u] = pfma(df, c_dr, pmul(sf, eC));
             if (rslab(i) && live) {
                 const uint32_t rx = rx_at(i) + u;
                 float2 *rq = rbuf + ((i & 1) * 4 + 2) * SLAB + u;
@@ -330,7 +330,7 @@ __global__ void __launch_bounds__(NT, NT > 192 ? 1 : 2) k_two(const __grid_const
                     q.oP[PS_EZ_R][rx] = w;
                 }
             }
-            tr[u] = pfma(psub(h.z.a[u], hz_j.a[u]), eA, pmul(dzp[u], c_ndz));
+            tr[u] = pfma(dzp[u], c_ndz, pmul(psub(h.z.a[u], hz_j.a[u]), eA));
             tz[u] = pfma(psub(h.r.a[u], hr_j.a[u]), eB, tz[u]);
         }
         float cr_[2] = {cn[0], cn[1]}, cp_[2] = {cn[0], cn[1]}, cz_[2] = {cc[0], cc[1]};
