@@ -59,8 +59,7 @@ def tune_zone(zone, steps=40, cache_path=None, use_cache=True):
     zone.default_kernel()
     own = zone.get_kernel()
     n0 = zone.launches
-    zone.time_steps(4)
-    one_launch = own[0] == 0 and zone.launches - n0 < 4
+    one_launch = own[0] == 0 and zone.time_steps(4) > 0 and zone.launches - n0 < 4
     # choices made without the one-launch run among them are not reused
     key = shape_key(zone.spec) + "_rpml%d" % zone.radial_pml() + ("_one_launch" if one_launch else "")
 

@@ -1744,6 +1744,7 @@ static zda_status time_steps_run(zda_zone *z, int steps, double *ms_out, cudaStr
 {
     zda_status st = ZDA_OK;
     z->have_forward = false;                 // the fields are overwritten
+    CUDA_TRY(cudaMemsetAsync(P<int>(*z, z->L.status) + 1, 0, sizeof(int), s));   // no timeout of an earlier run or owner
     zda::StepParams p = step_params(*z);
     p.src_mode = zda::SRC_NONE;
     p.mon = nullptr;
@@ -1779,7 +1780,6 @@ zda_status zda_zone_time_steps(zda_zone *z, int steps, double *ms_out, void *str
     if (steps < 1 || !ms_out) return fail(ZDA_ERR_ARG, "bad argument");
     st = time_steps_run(z, steps, ms_out, (cudaStream_t)stream, false);
     if (!repeat_by_split_step(*z, st)) return st;
-    CUDA_TRY(cudaMemsetAsync(P<int>(*z, z->L.status) + 1, 0, sizeof(int), (cudaStream_t)stream));
     return time_steps_run(z, steps, ms_out, (cudaStream_t)stream, true);
 }
 

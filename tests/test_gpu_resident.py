@@ -275,3 +275,13 @@ def test_a_tuned_small_zone_keeps_its_one_launch_run(tmp_path, name):
         n0 = t.launches
         t.forward(_dev(_rho(spec)))
         assert choice == (0, 2, 0) and t.launches - n0 < 20
+
+
+@pytest.mark.parametrize("kernel", [None, (0, 4, 0), (3, 8, 0), (4, 16, 0), (6, 16, 0)])
+def test_time_steps_reports_no_timeout_of_an_earlier_owner(kernel):
+    """The error word is whatever the workspace's memory held before, until a run clears it."""
+    z = _zone(_spec("tiny"))
+    if kernel:
+        z.set_kernel(*kernel)
+    z.workspace.fill_(1)                                 # (the tables are uploaded by the first run)
+    assert z.time_steps(4) > 0
