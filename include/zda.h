@@ -244,12 +244,13 @@ long long zda_zone_launch_count(const zda_zone *zone);
  * plan's estimate is below the split step's time (all but flat zones); else
  * variant 4 with 16 rows where it applies and the zone gives at least four
  * waves of its thread blocks (2 per SM) in radius ranges of about 21 radii;
- * else variant 0.  A zone with the default variant 0 whose whole field state
- * fits in the registers of one grid runs all its steps in one launch
- * instead (not under zda_zone_set_timing or the decay probe, not where
- * zones of a lens share the GPU, and not in a zda_forward of a zone of fine
- * cells or of few wavelengths, whose final fields have decayed to rounding
- * noise by its end).  Selecting
+ * else variant 0.  A zone with the default variant 0 whose whole state
+ * fits in the shared memory of one grid (at most four cells per thread) runs
+ * all its steps in one launch instead (not under zda_zone_set_timing or the
+ * decay probe, not where zones of a lens share the GPU or the stream is
+ * being captured, not for one step, and not in a zda_forward of a zone of
+ * fine cells or of few wavelengths, whose final fields may have decayed far
+ * below their peak).  Selecting
  * the stretched r-PML (form 1) on a zone that still has the default falls
  * back to variant 0, while an explicit variant 1, 3, 4, 5 or 6 refuses it.  All
  * compute the same scheme; results agree to FP32 rounding.  Variants 1, 3

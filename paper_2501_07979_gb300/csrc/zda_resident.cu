@@ -1,6 +1,6 @@
 // Resident time loop (sm_103a): every step of a small zone's run in one launch.
 //
-// What it is for: on a zone of up to about two hundred thousand cells the two
+// What it is for: on a zone of up to about three hundred thousand cells the two
 // or three launches of a split step cost 10-17 us, its arithmetic 1 us or so.
 // Here the zone is cut into bricks of cells, one thread block per brick and
 // SM, and a brick's state stays on its SM for the whole run: E and H in shared
@@ -10,7 +10,11 @@
 // optimisation iteration's time over its steps): 24 x 8 x 40 cells 10.4 us by
 // launches, 3.0 here; 248 x 1 x 160 (axis zone) 16.7 and 2.3; 48 x 48 x 64
 // 11.0 and 4.6; 64 x 50 x 64 17.5 and 8.5; 60 x 40 x 100 19.4 and 12.0.  So it
-// is taken wherever the zone fits (512 threads x 4 own cells per brick).
+// is taken wherever the zone fits (512 threads x 4 own cells per brick and its
+// state in the brick's shared memory), but where the launches of a step are
+// wanted or others share the GPU: a kernel chosen explicitly, event timing, the
+// decay probe, a lens, a stream capture, runs of one step, and forward runs
+// whose final fields may have decayed.
 //
 // What bounds it: small bricks the exchange (1.4 us of 2.3-3: a store to L2
 // and a load from it, across both dies); large ones shared-memory bandwidth,
